@@ -1,5 +1,7 @@
 // Total energy (Eq. 1 + Eq. 2, FP64) over the cell neighbourhoods, and the
 // time correlations of Sec. III.B (Eq. 5-7).
+#include <algorithm>
+
 #include "cell_list.h"
 #include "energy.h"
 #include "flipmc_device.cuh"
@@ -407,51 +409,127 @@ void launch_sq(const DevState &d, const long long *X, const double *qv, int n_q,
     sq_kernel<<<dim3(n_q, d.n_rep), 256, 0, st>>>(d, X, qv, n_q, out);
 }
 
-// Pair-distance histogram of one replica (Eq. gr): every pair once, by the
-// ring order: thread i takes the pairs (i, i + k mod N) for k = 1 .. (N-1)/2,
-// and for even N the pair (i, i + N/2) when i < N/2.  Bin = floor(r / dr)
-// with r from the FP64 minimum-image distance (each operation rounded once,
-// in a fixed order), counted when below n_bins.
-__global__ void __launch_bounds__(128) pair_hist_kernel(DevState d, const long long *X, double dr, int n_bins,
-                                                        unsigned long long *counts)
+// Pair-distance histogram (Eq. gr): counts[b] = pairs i < j with
+// floor(r / dr) = b, r from the FP64 minimum-image distance (each operation
+// rounded once, in a fixed order; pair_bin64 below).
+//
+// What bounds it: N^2 / 2 distances.  In FP64 each takes about 12 operations
+// of a pipe that does 2 per SM and cycle; a pass over the 2.9e8 pairs of 8000
+// molecules took 20.4 ms.  Here the bin comes from FP32 arithmetic on the
+// exact int32 differences, and FP64 decides only the pairs that FP32 cannot
+// place for certain: 0.44 ms for the same pass, bound by instruction issue (69%
+// of the slots, 42 instructions a pair).
+//
+// The FP32 value of f = r / dr is within 6.5 units of 2^-24 of its own size
+// (each difference rounds once when converted, three products and sums,
+// sqrt.approx within 2^-23, the factor h / dr and its product), so a value
+// further than 6e-7 f + 1e-6 (10 units) from a bin edge lies in the bin that
+// FP64 takes.  The others (one in some thousand) compare the exact integer
+// square D of the distance with the edge's, (e dr / h)^2 in FP64: both
+// decisions agree unless the two are within 17 units of 2^-53 of each other,
+// and inside 2^-45 the FP64 expression itself decides.
+//
+// Layout: blocks of 128 threads walk tile pairs of 128 x 128 records, one
+// record i per thread in registers, the records j broadcast from shared
+// memory.  The tile pairs of a replica are numbered by the ring distance d of
+// their tiles (p = d nt + ti, partner ti + d mod nt), which meets every
+// unordered pair of tiles once and needs no triangular root.  The histogram
+// stays in shared memory over all tile pairs of a block; up to 1024 bins it
+// is kept in four copies, by lane, because neighbouring lanes hit the same
+// few bins.
+constexpr int kHistTile = 128;
+constexpr int kHistCopyBins = 1024;          // up to so many bins: four copies (16 KB)
+constexpr int kHistBlocks = 152 * 12;        // blocks over all replicas (twelve per SM)
+
+// the bin of one pair in FP64 (may be >= n_bins)
+__device__ __noinline__ int pair_bin64(int dx, int dy, int dz, double h, double inv_h, double dr, int e)
 {
-    extern __shared__ unsigned int hist[];
-    const int r = blockIdx.y;
-    const RepInfo ri = d.rep[r];
-    const int N = ri.n_sites;
-    for (int b = threadIdx.x; b < n_bins; b += 128) hist[b] = 0;
-    __syncthreads();
-    const int i = blockIdx.x * 128 + threadIdx.x;
-    if (blockIdx.x * 128 < N) {
-        const double rmax = dr * (double)n_bins;
-        const double guard2 = rmax * rmax * (1.0 + 1e-12);
-        const int half = (N - 1) / 2;
-        const bool extra = (N % 2 == 0) && i < N / 2;
-        if (i < N) {
-            const long long *xi = X + 3 * (size_t)(ri.site_off + i);
-            const uint32_t ax = (uint32_t)xi[0], ay = (uint32_t)xi[1], az = (uint32_t)xi[2];
-            for (int k = 1; k <= half + (extra ? 1 : 0); ++k) {
-                int j = i + k;
-                if (j >= N) j -= N;
-                const long long *xj = X + 3 * (size_t)(ri.site_off + j);
-                const double r2 = r2_fixed64((int)((uint32_t)xj[0] - ax), (int)((uint32_t)xj[1] - ay),
-                                             (int)((uint32_t)xj[2] - az), ri.h);
-                if (!(r2 < guard2)) continue;
-                const int bin = (int)floor(__ddiv_rn(__dsqrt_rn(r2), dr));
-                if (bin < n_bins) atomicAdd(&hist[bin], 1u);
-            }
-        }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < n_bins; b += 128)
-        if (hist[b]) atomicAdd(counts + (size_t)r * n_bins + b, (unsigned long long)hist[b]);
+    const unsigned long long D = (unsigned long long)((long long)dx * dx) + (unsigned long long)((long long)dy * dy) +
+                                 (unsigned long long)((long long)dz * dz);
+    const double s = (double)e * dr * inv_h;
+    const double edge = s * s, diff = (double)D - edge;
+    if (fabs(diff) > edge * 0x1p-45) return diff > 0.0 ? e : e - 1;
+    return (int)floor(__ddiv_rn(__dsqrt_rn(r2_fixed64(dx, dy, dz, h)), dr));
 }
 
-void launch_pair_hist(const DevState &d, const long long *X, int max_sites, double dr, int n_bins,
-                      unsigned long long *counts, cudaStream_t st)
+template <int SH>
+__global__ void __launch_bounds__(kHistTile) pair_hist_kernel(DevState d, int buf, double dr, int n_bins,
+                                                              unsigned long long *counts)
 {
-    pair_hist_kernel<<<dim3((max_sites + 127) / 128, d.n_rep), 128, sizeof(unsigned int) * n_bins, st>>>(
-        d, X, dr, n_bins, counts);
+    extern __shared__ unsigned int hist[];   // n_bins << SH
+    __shared__ int4 tile[kHistTile];
+    const int r = blockIdx.y, tid = threadIdx.x;
+    const RepInfo ri = d.rep[r];
+    const int N = ri.n_sites;
+    const long long nt = (N + kHistTile - 1) / kHistTile, n_pairs = nt * (nt + 1) / 2;
+    if (blockIdx.x >= n_pairs) return;
+    const int4 *rec = d.rec[buf] + ri.site_off;
+    unsigned int *mine = hist + (tid & ((1 << SH) - 1));
+    for (int b = tid; b < n_bins << SH; b += kHistTile) hist[b] = 0;
+    const float scale = (float)fmin(ri.h / dr, 3.0e38);
+    auto flush = [&]() {
+        __syncthreads();
+        for (int b = tid; b < n_bins; b += kHistTile) {
+            unsigned long long v = 0;
+            for (int k = 0; k < 1 << SH; ++k) {
+                v += hist[(b << SH) + k];
+                hist[(b << SH) + k] = 0;
+            }
+            if (v) atomicAdd(counts + (size_t)r * n_bins + b, v);
+        }
+    };
+    unsigned done = 0;
+    for (long long p = blockIdx.x; p < n_pairs; p += gridDim.x) {
+        const int dist = (int)(p / nt), ti = (int)(p - dist * nt);
+        const int tj = (int)((ti + dist) % nt);
+        const int i = ti * kHistTile + tid, j0 = tj * kHistTile;
+        const int nj = min(kHistTile, N - j0);
+        __syncthreads();
+        if (tid < nj) tile[tid] = rec[j0 + tid];
+        __syncthreads();
+        const int4 me = rec[min(i, N - 1)];
+        // the first partner: every j of another tile, the later ones of its own
+        const int first = i >= N ? nj : (dist == 0 ? tid + 1 : 0);
+#pragma unroll 4
+        for (int j = 0; j < nj; ++j) {
+            const int4 o = tile[j];
+            const int dx = (int)((uint32_t)o.x - (uint32_t)me.x), dy = (int)((uint32_t)o.y - (uint32_t)me.y),
+                      dz = (int)((uint32_t)o.z - (uint32_t)me.z);
+            const float fx = (float)dx, fy = (float)dy, fz = (float)dz;
+            float root;
+            asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(fx, fx, fmaf(fy, fy, fz * fz))));
+            // bin = round(f - 1/2) by the exponent trick: 1.5 x 2^23 + g rounds
+            // g to an integer, which then stands in the low bits (for g of
+            // 2^22 and more, a value that exceeds every n_bins)
+            const float g = fmaf(root, scale, -0.5f);
+            const float t = g + 12582912.0f;
+            const float off = g - (t - 12582912.0f);
+            int bin = __float_as_int(t) - 0x4B400000;
+            if (j >= first && bin <= n_bins) {
+                if (fabsf(off) > fmaf(-6e-7f, g, 0.499999f))
+                    bin = pair_bin64(dx, dy, dz, ri.h, ri.inv_h, dr, off > 0.f ? bin + 1 : bin);
+                if (bin < n_bins) atomicAdd(mine + (bin << SH), 1u);
+            }
+        }
+        // a 32-bit count takes at most 2^17 tile pairs of 2^14 pairs
+        if (++done == 1u << 17) {
+            flush();
+            done = 0;
+        }
+    }
+    flush();
+}
+
+void launch_pair_hist(const DevState &d, int buf, int max_sites, double dr, int n_bins, unsigned long long *counts,
+                      cudaStream_t st)
+{
+    const long long nt = (max_sites + kHistTile - 1) / kHistTile, n_pairs = nt * (nt + 1) / 2;
+    const long long bx = std::min<long long>(n_pairs, std::max(1, kHistBlocks / d.n_rep));
+    const dim3 grid((unsigned)bx, d.n_rep);
+    if (n_bins <= kHistCopyBins)
+        pair_hist_kernel<2><<<grid, kHistTile, sizeof(unsigned int) * 4 * n_bins, st>>>(d, buf, dr, n_bins, counts);
+    else
+        pair_hist_kernel<0><<<grid, kHistTile, sizeof(unsigned int) * n_bins, st>>>(d, buf, dr, n_bins, counts);
 }
 
 void launch_gather(const DevState &d, int buf, long long *X, int *types, cudaStream_t st)

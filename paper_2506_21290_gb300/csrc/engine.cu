@@ -1116,8 +1116,7 @@ int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, dou
     CUDA_TRY(cudaMallocAsync(&dc, sizeof(unsigned long long) * n, h->stream));
     cudaError_t e = cudaMemsetAsync(dc, 0, sizeof(unsigned long long) * n, h->stream);
     if (e == cudaSuccess) {
-        launch_gather(h->ds, h->cur, h->d_X, h->d_types, h->stream);
-        launch_pair_hist(h->ds, h->d_X, max_sites, dr, n_bins, dc, h->stream);
+        launch_pair_hist(h->ds, h->cur, max_sites, dr, n_bins, dc, h->stream);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
