@@ -23,9 +23,11 @@
  * are Philox4x32-10 keyed on (seed) and counted on (attempt, cell, sweep), so a
  * run is reproducible bit for bit and independent of the launch layout.
  *
- * Precision.  MC_PREC_FP64 evaluates every Delta E in FP64 with one rounding per
- * operation, summed in a fixed order (moved atom ascending, then partner index
- * ascending); it reproduces the library's FP64 reference trajectory exactly.
+ * Precision.  MC_PREC_FP64 decides every attempt as Delta E in FP64 with one
+ * rounding per operation, summed in a fixed order (moved atom ascending, then
+ * partner index ascending), does; it reproduces the library's FP64 reference
+ * trajectory, running energy and counters exactly.  An attempt that a rigorous
+ * FP32 bound refuses is refused without the sum (a logged sweep sums them all).
  * MC_PREC_FP32 evaluates pair terms in FP32 and decides in FP32 when
  * |dE32 - threshold| exceeds recheck_gap times the sum of term magnitudes plus
  * the threshold's own error bound (the FP32 decision then equals the FP64 one);

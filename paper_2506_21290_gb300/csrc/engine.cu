@@ -248,6 +248,18 @@ void build_model(const mc_params &p, double gap, ModelDev &md)
     md.recheck_gap_f = (float)gap;
 }
 
+// Whether the FP32 error bound of the sweeps holds over the whole range of a
+// potential and a box: it is relative to term magnitudes of at least eps or
+// K eps, so these, the squared diameters and the squared quantum have to be
+// normal FP32 numbers with room for products.
+bool fp32_bound_holds(const ModelDev &md, double L)
+{
+    auto normal = [](double x) { return x > 1e-20 && x < 1e20; };
+    bool ok = normal(md.eps) && (md.ke == 0.0 || normal(md.ke)) && L > 1e-6 && L < 1e6;
+    for (int k = 0; k < 9; ++k) ok = ok && normal(md.s2[k]) && normal(md.R2[k]);
+    return ok;
+}
+
 // Longest interaction range: the WCA cutoff of any type pair, and the FENE
 // divergence of any pair that can form a bond (type pairs inside a molecule's
 // multiset, which flips permute but never change).
@@ -571,6 +583,7 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         ri.inv_h = kTwo32 / L[r];
         ri.hf = (float)ri.h;
         ri.h2f = (float)(ri.h * ri.h);
+        ri.filter64 = fp32_bound_holds(h->model_host, L[r]);
         // the radii of the screens and of the conflict test, in FP32 as the
         // kernels use them (one rounding per operation)
         float rc2max = 0.f;

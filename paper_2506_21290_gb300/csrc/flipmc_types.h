@@ -32,7 +32,7 @@ struct RepInfo {
     int nc;          // cells per axis
     int cell_off;    // first global cell
     int act_off;     // first global active-cell slot within a colour
-    int pad;
+    int filter64;    // FP64 mode may refuse attempts by FP32 arithmetic: its terms stay in FP32's normal range
     double L, h, inv_h;
     float hf;
     float h2f;       // h^2 rounded to FP32

@@ -38,12 +38,28 @@
 // a padding record, discarded queue writes go to a spare slot, and terms are
 // masked instead of skipped.
 //
-// FP64 mode: every Delta E is the FP64 ordered sum (moved atom ascending, then
-// partner index ascending) of the nonzero pair terms, each operation unfused
-// and rounded to nearest, and the threshold is the FP64 series logarithm; this
-// reproduces the reference FP64 chain exactly.  The terms are taken over the
-// queued partners only: the screening radius exceeds every cutoff by far more
-// than the FP32 distance error, so every partner with a nonzero term is queued.
+// FP64 mode: every Delta E that decides an attempt or enters the running total
+// or the log is the FP64 ordered sum (moved atom ascending, then partner index
+// ascending) of the nonzero pair terms, each operation unfused and rounded to
+// nearest, and the threshold is the FP64 series logarithm; this reproduces the
+// reference FP64 chain exactly.  The terms are taken over the queued partners
+// only: the screening radius exceeds every cutoff by far more than the FP32
+// distance error, so every partner with a nonzero term is queued.
+//
+// The FP64 sum is the long part of an attempt (a dependent FP64 add takes 64
+// cycles here and a division 564), and nine attempts in ten are refused far
+// from the threshold.  So FP64 mode first runs the FP32 pass of step 2 with
+// the margin of step 3 (never below 1e-5, whatever the handle's recheck_gap):
+// an attempt that it refuses for certain is refused without the sum.  Every
+// other attempt (accepted, near the threshold, a bond near its divergence, a
+// pair within 2e-6 of its cutoff, whose place in the pair_interactions count
+// FP32 cannot tell) takes the sum and is decided by it, and a logged sweep
+// takes it for all.  Decisions, running totals, counts and logs are those of
+// the sum for every attempt.  20 sweeps of 8000 molecules with
+// energy and read-back: 8.51 -> 3.87 ms (3.25 ms with the sum itself in tasks,
+// dE64_ordered).
+// The bound needs FP32's normal range, so parameters far from it (filter64 of
+// the replica, and T) keep the sum for every attempt.
 #include <algorithm>
 #include <cstdio>
 
@@ -186,9 +202,8 @@ __device__ __forceinline__ void bulk_to_smem(void *dst, const void *src, unsigne
 // per warp: interaction queue, and (aliased, used after it) the FP64 term buffers
 struct WarpScr {
     int *qc;                    // [QW + 1] queued candidate indices, then a slot that takes discarded writes
-    unsigned long long *key;    // [TERM_CAP] term keys; after ranking, the values in key order (as doubles)
+    unsigned long long *key;    // [TERM_CAP] tasks and term keys; after ranking, the values in key order (as doubles)
     double *val;                // [TERM_CAP]
-    int *cnt;                   // [4]
 };
 
 // the outcome of one evaluated attempt (registers of the evaluating warp,
@@ -253,7 +268,7 @@ __host__ __device__ constexpr size_t warp_scr_bytes()
     return (al16(sizeof(int) * (QW + 1)) > al16(sizeof(unsigned long long) * TERM_CAP)
                 ? al16(sizeof(int) * (QW + 1))
                 : al16(sizeof(unsigned long long) * TERM_CAP)) +
-           al16(sizeof(double) * TERM_CAP) + al16(sizeof(int) * 4);
+           al16(sizeof(double) * TERM_CAP);
 }
 
 // Layout of a group's shared memory: the fixed-size parts first (at offsets
@@ -303,7 +318,6 @@ __device__ inline WarpScr warp_scr(const Group &G, int wig)
     s.qc = (int *)b;
     s.key = (unsigned long long *)b;    // aliases the queue: used only after it
     s.val = (double *)(b + qk);
-    s.cnt = (int *)(b + qk + al16(sizeof(double) * TERM_CAP));
     return s;
 }
 
@@ -341,7 +355,6 @@ struct Move {
     uint32_t qo[3][3];     // old positions
     uint32_t qn[3][3];     // new positions
     int to[3], tn[3];      // old / new types
-    bool moves_pos;
     bool intra;            // rotation: intramolecular pairs change too
 };
 
@@ -354,90 +367,138 @@ struct Move {
 // atom of the molecule, so no nonzero term is missed), else all K staged atoms.
 // Terms are keyed by (moved atom, partner site), so which lane computes a term
 // does not change the sum.
+//
+// What bounds it is latency: a dependent FP64 operation takes 64 cycles and a
+// division 564, so a pair's old and new terms one after the other, with the
+// logarithms of the bonds in between, were a chain of about 7000 cycles.  Here
+// every potential of the move is a task of its own: the Eq. 1 value of a pair
+// in one configuration (only pairs that FP32 places inside their cutoff, with
+// a margin; the others are exactly 0), and the Eq. 2 value of a bond in one
+// configuration.  A move has about 23 tasks, so one batch of 32 lanes does all
+// of them at once; both kinds share the first division (sigma^2 / r^2 and
+// r^2 / R0^2 sigma^2), and the Eq. 1 products run under the logarithm.  The
+// lane that holds a pair then fetches its values and forms
+// (u_new + fene_new) - (u_old + fene_old) with the roundings of phi64.
+// Five FP64 sweeps of 64 molecules (a quarter of the attempts accepted): 2.48 ->
+// 1.97 ms; twenty of 8000: 3.87 -> 3.25 ms.  The FP32 chain, which takes the sum
+// only near a threshold, gains 3-4% because one slow attempt holds its round.
+constexpr int kTaskOld = 0, kTaskNew = 1, kTaskFene = 2;   // bit 0 configuration, bit 1 potential
+
 __device__ __noinline__ int dE64_ordered(const Move &mv, const RecView rv, const WarpScr S, int K, int nq,
-                                         const ModelDev &md, double h, float hf, float pre_r2, int lane, int *err,
-                                         double &dE, int &inter)
+                                         const ModelDev &md, double h, float hf, int lane, int *err, double &dE,
+                                         int &inter)
 {
     inter = 0;
     static_assert(QW <= 64, "a lane takes at most two queue entries");
+    static_assert(TERM_CAP == 128, "tasks (256 halfwords), then keys (128 words), fill the key array");
+    unsigned short *task = (unsigned short *)S.key;
+    unsigned *key = (unsigned *)S.key + 128;
+    const unsigned lt = (1u << lane) - 1u;
     // the term buffers alias the queue: take the entries into registers first
-    int qe0 = -1, qe1 = -1;
+    int ent[2] = {-1, -1};
     if (nq >= 0) {
-        if (lane < nq) qe0 = S.qc[lane];
-        if (lane + 32 < nq) qe1 = S.qc[lane + 32];
+        if (lane < nq) ent[0] = S.qc[lane];
+        if (lane + 32 < nq) ent[1] = S.qc[lane + 32];
     }
     __syncwarp();
-    if (lane == 0) S.cnt[0] = 0;
-    __syncwarp();
-    int brk = 0;
-    auto term_of = [&](int c) {
-        const int4 r = rv.at(c);
-        const int sj = rec_site(r.w);
-        bool in_set = false;
-        for (int k = 0; k < mv.n; ++k) in_set |= (sj == mv.site[k]);
-        if (in_set) return;
-        const bool bonded = rec_mol(r.w) == mv.mol;
-        const int tj = rec_type(r.w);
-        for (int k = 0; k < mv.n; ++k) {
-            const int dxo = (int)((uint32_t)r.x - mv.qo[k][0]);
-            const int dyo = (int)((uint32_t)r.y - mv.qo[k][1]);
-            const int dzo = (int)((uint32_t)r.z - mv.qo[k][2]);
-            const int dxn = (int)((uint32_t)r.x - mv.qn[k][0]);
-            const int dyn = (int)((uint32_t)r.y - mv.qn[k][1]);
-            const int dzn = (int)((uint32_t)r.z - mv.qn[k][2]);
-            if (!bonded) {
-                // conservative FP32 screen: a pair beyond every cutoff adds exactly 0
-                const float fxo = (float)dxo * hf, fyo = (float)dyo * hf, fzo = (float)dzo * hf;
-                const float fxn = (float)dxn * hf, fyn = (float)dyn * hf, fzn = (float)dzn * hf;
-                const float r2of = fxo * fxo + fyo * fyo + fzo * fzo;
-                const float r2nf = fxn * fxn + fyn * fyn + fzn * fzn;
-                if (r2of > pre_r2 && r2nf > pre_r2) continue;
-            }
-            const double r2o = r2_fixed64(dxo, dyo, dzo, h);
-            const double r2n = mv.moves_pos ? r2_fixed64(dxn, dyn, dzn, h) : r2o;
-            const int abo = 3 * mv.to[k] + tj, abn = 3 * mv.tn[k] + tj;
-            inter += (r2o < md.rc2[abo]) + (r2n < md.rc2[abn]) + (bonded ? 2 : 0);
-            if (bonded && !(r2n < md.R2[abn])) brk = 1;
-            const double term = __dsub_rn(phi64(md, r2n, abn, bonded), phi64(md, r2o, abo, bonded));
-            if (term != 0.0) {
-                const int p = atomicAdd(S.cnt, 1);
-                if (p < TERM_CAP) {
-                    S.key[p] = ((unsigned long long)k << 32) | (unsigned)sj;
-                    S.val[p] = term;
-                }
-            }
+    int nt = 0, brk = 0;
+    // append the lanes' nonzero terms
+    auto push = [&](bool live, unsigned k, double term) {
+        const bool nz = live && term != 0.0;
+        const unsigned b = __ballot_sync(FULL, nz);
+        const int p = nt + __popc(b & lt);
+        if (nz && p < TERM_CAP) {
+            key[p] = k;
+            S.val[p] = term;
         }
+        nt += __popc(b);
     };
-    if (nq >= 0) {
-        if (qe0 >= 0) term_of(qe0);
-        if (qe1 >= 0) term_of(qe1);
-    } else {
-        for (int c = lane; c < K; c += 32) term_of(c);
-    }
-    if (mv.intra && lane == 0) {
-        const int pk3[3] = {0, 0, 1}, pl3[3] = {1, 2, 2};
-        for (int pr = 0; pr < 3; ++pr) {
-            const int k = pk3[pr], l = pl3[pr];
-            const int ab = 3 * mv.to[k] + mv.to[l];
-            const double r2o = r2_fixed64((int)(mv.qo[l][0] - mv.qo[k][0]), (int)(mv.qo[l][1] - mv.qo[k][1]),
-                                          (int)(mv.qo[l][2] - mv.qo[k][2]), h);
-            const double r2n = r2_fixed64((int)(mv.qn[l][0] - mv.qn[k][0]), (int)(mv.qn[l][1] - mv.qn[k][1]),
-                                          (int)(mv.qn[l][2] - mv.qn[k][2]), h);
-            inter += (r2o < md.rc2[ab]) + (r2n < md.rc2[ab]) + 2;
-            if (!(r2n < md.R2[ab])) brk = 1;
-            const double term = __dsub_rn(phi64(md, r2n, ab, true), phi64(md, r2o, ab, true));
-            if (term != 0.0) {
-                const int p = atomicAdd(S.cnt, 1);
-                if (p < TERM_CAP) {
-                    S.key[p] = (3ull << 32) | (unsigned)pr;
-                    S.val[p] = term;
+    // 32 candidates at a time: the queue's, or all the staged atoms
+    const int n_cand = nq >= 0 ? nq : K;
+#pragma unroll 1
+    for (int c0 = 0; c0 < n_cand; c0 += 32) {
+        const int cand = c0 + lane >= n_cand ? -1 : (nq < 0 ? c0 + lane : (c0 == 0 ? ent[0] : ent[1]));
+#pragma unroll 1
+        for (int k = 0; k < mv.n; ++k) {
+            const int to = mv.to[k], tn = mv.tn[k];
+            const uint32_t *qo = mv.qo[k], *qn = mv.qn[k];
+            bool live = cand >= 0, bond = false;
+            int site = 0, n_task = 0, pos[4] = {-1, -1, -1, -1};
+            {
+                const int4 r = rv.at(max(cand, 0));
+                site = rec_site(r.w);
+                for (int m = 0; m < mv.n; ++m) live = live && site != mv.site[m];
+                bond = live && rec_mol(r.w) == mv.mol;
+                auto near = [&](const uint32_t *q, int ab) {
+                    const float fx = dq((uint32_t)r.x, q[0]) * hf, fy = dq((uint32_t)r.y, q[1]) * hf,
+                                fz = dq((uint32_t)r.z, q[2]) * hf;
+                    return live && fx * fx + fy * fy + fz * fz <= md.rc2f[ab] * 1.00001f;
+                };
+                const int tj = rec_type(r.w);
+                const bool want[4] = {near(qo, 3 * to + tj), near(qn, 3 * tn + tj), bond, bond};
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const unsigned b = __ballot_sync(FULL, want[j]);
+                    if (want[j]) {
+                        pos[j] = n_task + __popc(b & lt);
+                        task[pos[j]] = (unsigned short)(cand << 2 | j);
+                    }
+                    n_task += __popc(b);
                 }
             }
+            __syncwarp();
+            double u[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+            for (int t0 = 0; t0 < n_task; t0 += 32) {
+                const bool on = t0 + lane < n_task;
+                const int t = on ? task[t0 + lane] : 0;
+                const bool fene = on && (t & kTaskFene), fresh = (t & kTaskNew) != 0;
+                const int4 r = rv.at(t >> 2);
+                const int ab = 3 * (fresh ? tn : to) + rec_type(r.w);
+                const uint32_t *q = fresh ? qn : qo;
+                double r2 = r2_fixed64((int)((uint32_t)r.x - q[0]), (int)((uint32_t)r.y - q[1]),
+                                       (int)((uint32_t)r.z - q[2]), h);
+                if (!on) r2 = 1.0;
+                const bool in = r2 < md.rc2[ab];
+                if (fene && fresh && !(r2 < md.R2[ab])) brk = 1;
+                inter += on && (fene || in);
+                const double ratio = __ddiv_rn(fene ? r2 : md.s2[ab], fene ? md.R2[ab] : r2);
+                const double s6 = __dmul_rn(__dmul_rn(ratio, ratio), ratio);
+                double v = __dadd_rn(__dmul_rn(md.e4, __dsub_rn(__dmul_rn(s6, s6), s6)), md.eps);
+                if (!in) v = 0.0;
+                if (__any_sync(FULL, fene)) {
+                    const double f = __dmul_rn(md.nke, ln_series(__dsub_rn(1.0, fene ? ratio : 0.0)));
+                    if (fene) v = f;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const double g = __shfl_sync(FULL, v, pos[j] & 31);
+                    if (pos[j] >> 5 == t0 >> 5) u[j] = g;
+                }
+            }
+            if (bond) {
+                u[0] = __dadd_rn(u[0], u[2]);
+                u[1] = __dadd_rn(u[1], u[3]);
+            }
+            push(live, (unsigned)k << 29 | (unsigned)site, __dsub_rn(u[1], u[0]));
+            __syncwarp();
         }
+    }
+    if (mv.intra) {
+        // the three pairs of the molecule, old in lanes 0-2, new in lanes 3-5
+        const int pr = lane % 3, k = pr == 2 ? 1 : 0, l = pr == 0 ? 1 : 2;
+        const bool on = lane < 6, fresh = lane >= 3;
+        const int ab = 3 * mv.to[k] + mv.to[l];
+        const uint32_t(*q)[3] = fresh ? mv.qn : mv.qo;
+        const double r2 = on ? r2_fixed64((int)(q[l][0] - q[k][0]), (int)(q[l][1] - q[k][1]), (int)(q[l][2] - q[k][2]), h)
+                             : 1.0;
+        const double v = on ? phi64(md, r2, ab, true) : 0.0;
+        inter += on ? (r2 < md.rc2[ab]) + 1 : 0;
+        if (on && fresh && !(r2 < md.R2[ab])) brk = 1;
+        const double vn = __shfl_down_sync(FULL, v, 3);
+        push(lane < 3, 3u << 29 | (unsigned)pr, __dsub_rn(vn, v));
     }
     brk = __any_sync(FULL, brk);
-    __syncwarp();
-    const int nt = S.cnt[0];
     if (nt > TERM_CAP) {
         if (lane == 0) atomicOr(err, ERR_TERMS);
         dE = __longlong_as_double(0x7FF8000000000000ll);
@@ -445,20 +506,22 @@ __device__ __noinline__ int dE64_ordered(const Move &mv, const RecView rv, const
     }
     // rank every term by its key (keys are distinct), then put the values in
     // key order over the key array and sum them in that order
-    static_assert(TERM_CAP <= 128, "a lane ranks at most four terms");
-    unsigned long long kk[4];
+    if (lane < 4 && nt + lane < TERM_CAP) key[nt + lane] = ~0u;   // whole quads below
+    __syncwarp();
+    unsigned kk[4];
     double vv[4];
     int rk[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
         const int e = lane + 32 * s;
-        kk[s] = e < nt ? S.key[e] : ~0ull;
+        kk[s] = e < nt ? key[e] : ~0u;
         vv[s] = e < nt ? S.val[e] : 0.0;
     }
-    for (int f = 0; f < nt; ++f) {
-        const unsigned long long kf = S.key[f];
+    for (int f = 0; f < nt; f += 4) {
+        const uint4 kf = *(const uint4 *)(key + f);
 #pragma unroll
-        for (int s = 0; s < 4; ++s) rk[s] += kf < kk[s];
+        for (int s = 0; s < 4; ++s)
+            if (32 * s < nt) rk[s] += (kf.x < kk[s]) + (kf.y < kk[s]) + (kf.z < kk[s]) + (kf.w < kk[s]);
     }
     __syncwarp();
     double *sorted = (double *)S.key;
@@ -466,10 +529,10 @@ __device__ __noinline__ int dE64_ordered(const Move &mv, const RecView rv, const
     for (int s = 0; s < 4; ++s)
         if (lane + 32 * s < nt) sorted[rk[s]] = vv[s];
     __syncwarp();
-    double s = 0.0;
-    if (lane == 0)
-        for (int e = 0; e < nt; ++e) s = __dadd_rn(s, sorted[e]);
-    dE = __shfl_sync(FULL, s, 0);
+    // (every lane the same sum; no term is 0, so the first one is 0 + itself)
+    double sum = nt > 0 ? sorted[0] : 0.0;
+    for (int e = 1; e < nt; ++e) sum = __dadd_rn(sum, sorted[e]);
+    dE = sum;
     __syncwarp();
     return brk ? MC_ST_BOND_BREAK : MC_ST_EVALUATED;
 }
@@ -708,8 +771,15 @@ struct Acc32 {
     int cnt;                    // pair-potential evaluations inside their range
 };
 
+// EDGE: a pair whose FP32 distance may lie on the other side of the cutoff than
+// its FP64 one (r^2 is within 9 units of 2^-24, rc^2 within one) raises the
+// guard, so that without a guard the count is the FP64 one.
+__device__ __forceinline__ bool near_cutoff(float r2, float rc2) { return fabsf(r2 - rc2) <= 2e-6f * rc2; }
+
+template <bool EDGE>
 __device__ __forceinline__ void add_wca(const ModelDev &md, float r2, int ab, float sign, Acc32 &a)
 {
+    if (EDGE && near_cutoff(r2, md.rc2f[ab])) a.guard = 1;
     if (r2 < md.rc2f[ab]) {
         float u, m;
         wca32(md, r2, ab, u, m);
@@ -736,11 +806,13 @@ __device__ __forceinline__ void add_fene(const ModelDev &md, float r2, int ab, f
 // multiplies it by 0 or 1, so the warp never diverges (in a latency-bound warp
 // a divergent branch costs more than the arithmetic it skips).  Terms that are
 // on add exactly what add_wca / add_fene add.
+template <bool EDGE>
 __device__ __forceinline__ void wca_m(const ModelDev &md, float r2, int ab, float sign, Acc32 &a)
 {
     float u, m;
     wca32(md, r2, ab, u, m);
     const bool in = r2 < md.rc2f[ab];
+    if (EDGE) a.guard |= near_cutoff(r2, md.rc2f[ab]);
     const float on = in ? 1.f : 0.f;
     a.dE = fmaf(sign * on, u, a.dE);
     a.mag = fmaf(on, m, a.mag);
@@ -777,6 +849,7 @@ __device__ __forceinline__ int queued(const WarpScr &S, int e, int nq, int K, in
     return (e < nq && cq != k0 && cq != k1) ? cq : K;
 }
 
+template <bool EDGE>
 __device__ __forceinline__ Acc32 inter_atom(const Group &G, const WarpScr &S, int nq, int lane, const ModelDev &md,
                                             int K, int k, int wi, int ti, const Q3 &qo, const Q3 &qn, float h2)
 {
@@ -789,8 +862,8 @@ __device__ __forceinline__ Acc32 inter_atom(const Group &G, const WarpScr &S, in
             const int ab = 3 * ti + rec_type(r.w);
             const bool bonded = (r.w ^ wi) < 16;
             const float r2o = cand_r2(r, qo, h2), r2n = cand_r2(r, qn, h2);
-            wca_m(md, r2o, ab, -1.f, a);
-            wca_m(md, r2n, ab, 1.f, a);
+            wca_m<EDGE>(md, r2o, ab, -1.f, a);
+            wca_m<EDGE>(md, r2n, ab, 1.f, a);
             fene_m(md, r2o, ab, -1.f, bonded, a);
             fene_m(md, r2n, ab, 1.f, bonded, a);
         }
@@ -798,6 +871,7 @@ __device__ __forceinline__ Acc32 inter_atom(const Group &G, const WarpScr &S, in
     return a;
 }
 
+template <bool EDGE>
 __device__ __forceinline__ Acc32 inter_flip(const Group &G, const WarpScr &S, int nq, int lane, const ModelDev &md,
                                             int K, int kp, int kq, int wi, int tp, int tq, const Q3 &qp,
                                             const Q3 &qq, float h2)
@@ -812,10 +886,10 @@ __device__ __forceinline__ Acc32 inter_flip(const Group &G, const WarpScr &S, in
             const bool bonded = (r.w ^ wi) < 16;
             const float rp = cand_r2(r, qp, h2), rq = cand_r2(r, qq, h2);
             // atom p: type tp -> tq; atom q: type tq -> tp
-            wca_m(md, rp, 3 * tp + tj, -1.f, a);
-            wca_m(md, rp, 3 * tq + tj, 1.f, a);
-            wca_m(md, rq, 3 * tq + tj, -1.f, a);
-            wca_m(md, rq, 3 * tp + tj, 1.f, a);
+            wca_m<EDGE>(md, rp, 3 * tp + tj, -1.f, a);
+            wca_m<EDGE>(md, rp, 3 * tq + tj, 1.f, a);
+            wca_m<EDGE>(md, rq, 3 * tq + tj, -1.f, a);
+            wca_m<EDGE>(md, rq, 3 * tp + tj, 1.f, a);
             fene_m(md, rp, 3 * tp + tj, -1.f, bonded, a);
             fene_m(md, rp, 3 * tq + tj, 1.f, bonded, a);
             fene_m(md, rq, 3 * tq + tj, -1.f, bonded, a);
@@ -825,6 +899,7 @@ __device__ __forceinline__ Acc32 inter_flip(const Group &G, const WarpScr &S, in
     return a;
 }
 
+template <bool EDGE>
 __device__ __noinline__ Acc32 inter_mol(const Group G, const WarpScr S, int nq, int lane, const ModelDev &md, int K,
                                         const int *t3, const Q3 *qo, const Q3 *qn, float h2)
 {
@@ -834,14 +909,15 @@ __device__ __noinline__ Acc32 inter_mol(const Group G, const WarpScr S, int nq, 
         const int tj = rec_type(r.w);
         for (int m = 0; m < 3; ++m) {
             const int ab = 3 * t3[m] + tj;
-            wca_m(md, cand_r2(r, qo[m], h2), ab, -1.f, a);
-            wca_m(md, cand_r2(r, qn[m], h2), ab, 1.f, a);
+            wca_m<EDGE>(md, cand_r2(r, qo[m], h2), ab, -1.f, a);
+            wca_m<EDGE>(md, cand_r2(r, qn[m], h2), ab, 1.f, a);
         }
     }
     return a;
 }
 
 // intramolecular terms of a rotation (FP32, one lane), added to part
+template <bool EDGE>
 __device__ __noinline__ Acc32 rot_intra32(const ModelDev &md, const Q3 *qo, const Q3 *qn, const int *t3, float hf,
                                           Acc32 part)
 {
@@ -853,8 +929,8 @@ __device__ __noinline__ Acc32 rot_intra32(const ModelDev &md, const Q3 *qo, cons
         const int4 rn = make_int4((int)qn[ll].x, (int)qn[ll].y, (int)qn[ll].z, 0);
         const float r2o = r2_int32f(ro, qo[kk], hf);
         const float r2n = r2_int32f(rn, qn[kk], hf);
-        add_wca(md, r2o, ab, -1.f, part);
-        add_wca(md, r2n, ab, 1.f, part);
+        add_wca<EDGE>(md, r2o, ab, -1.f, part);
+        add_wca<EDGE>(md, r2n, ab, 1.f, part);
         add_fene(md, r2o, ab, -1.f, part);
         add_fene(md, r2n, ab, 1.f, part);
     }
@@ -873,9 +949,9 @@ struct CellCtx {
     uint32_t shift[3];
     double h, inv_h, T64;
     float hf, h2f;          // h and h^2 in FP32
-    float pre_r2;           // screening radius squared (sigma units): 1.01 x the largest WCA cutoff squared
-    float r2q;              // the same in fixed-point units squared (the screens' units)
+    float r2q;              // screening radius squared, fixed-point units: 1.01 x the largest WCA cutoff squared
     float gap, T32;
+    bool filter;            // FP64 mode: attempts may be refused by the FP32 pass
     int *err;
 };
 
@@ -887,8 +963,9 @@ __device__ __forceinline__ PosH local_of(const CellCtx &c, const Q3 &q)
 // Evaluate attempt `jr` of the current chunk (one warp, state read-only) and
 // return its outcome (the same in every lane); with W > 1 lane 0 also leaves
 // in N what the conflict test of the later attempts of the round reads.
+// all_sums (FP64 mode): the FP64 sum for every attempt (the attempts are logged).
 template <int PREC, int W>
-__device__ Res evaluate(const CellCtx &cx, const Group &G, const WarpScr &S, Near *N, int jr, int lane)
+__device__ Res evaluate(const CellCtx &cx, const Group &G, const WarpScr &S, Near *N, int jr, int lane, bool all_sums)
 {
     const ModelDev &md = *cx.md;
     // the attempt's draws, decoded by the cell-list build (site rank, move type,
@@ -991,7 +1068,6 @@ __device__ Res evaluate(const CellCtx &cx, const Group &G, const WarpScr &S, Nea
         Move mv;
         mv.n = nmv;
         mv.mol = mol;
-        mv.moves_pos = mvt != MC_MOVE_FLIP;
         mv.intra = mvt == MC_MOVE_MOL_ROT;
 #pragma unroll
         for (int s = 0; s < 3; ++s) {
@@ -1007,7 +1083,7 @@ __device__ Res evaluate(const CellCtx &cx, const Group &G, const WarpScr &S, Nea
         }
         double e64 = 0.0;
         int cnt64 = 0;
-        const int st = dE64_ordered(mv, cx.rv, S, K, nq, md, cx.h, cx.hf, cx.pre_r2, lane, cx.err, e64, cnt64);
+        const int st = dE64_ordered(mv, cx.rv, S, K, nq, md, cx.h, cx.hf, lane, cx.err, e64, cnt64);
         dE64 = e64;
         if (PREC == MC_PREC_FP64) inter = cnt64;
         return (st == MC_ST_EVALUATED) ? ((e64 <= thr) ? 1 : 0) : -1;
@@ -1026,24 +1102,44 @@ __device__ Res evaluate(const CellCtx &cx, const Group &G, const WarpScr &S, Nea
         __syncwarp();
         const int nq = min(qlen, QW);
         const int nq64 = qlen <= QW ? qlen : -1;   // overflowed queue: the FP64 sum scans every atom
-        if (PREC == MC_PREC_FP64) {
-            const int dec = exact(G.thr64[jr], nq64);
-            if (dec < 0) status = MC_ST_BOND_BREAK;
-            accept = dec == 1;
-        } else {
-            const float thr32 = G.thr32[jr];
+        // the FP32 pass over the queue: this lane's share
+        auto pass32 = [&]() {
+            constexpr bool EDGE = PREC == MC_PREC_FP64;
             Acc32 part;
             if (mvt == MC_MOVE_ATOM) {
-                part = inter_atom(G, S, nq, lane, md, K, k, wi, t3o[0], qo[0], qn[0], cx.h2f);
+                part = inter_atom<EDGE>(G, S, nq, lane, md, K, k, wi, t3o[0], qo[0], qn[0], cx.h2f);
             } else if (mvt == MC_MOVE_FLIP) {
-                part = inter_flip(G, S, nq, lane, md, K, ks[0], ks[1], wi, t3o[0], t3o[1], qo[0], qo[1], cx.h2f);
+                part = inter_flip<EDGE>(G, S, nq, lane, md, K, ks[0], ks[1], wi, t3o[0], t3o[1], qo[0], qo[1], cx.h2f);
             } else {
                 const int tm[3] = {t3o[0], t3o[1], t3o[2]};
                 const Q3 ro[3] = {qo[0], qo[1], qo[2]}, rn[3] = {qn[0], qn[1], qn[2]};
-                part = inter_mol(G, S, nq, lane, md, K, tm, ro, rn, cx.h2f);
-                if (mvt == MC_MOVE_MOL_ROT && lane == 0) part = rot_intra32(md, ro, rn, tm, cx.hf, part);
+                part = inter_mol<EDGE>(G, S, nq, lane, md, K, tm, ro, rn, cx.h2f);
+                if (mvt == MC_MOVE_MOL_ROT && lane == 0) part = rot_intra32<EDGE>(md, ro, rn, tm, cx.hf, part);
             }
             if (qlen > QW) part.guard = 1;
+            return part;
+        };
+        if (PREC == MC_PREC_FP64) {
+            bool refused = false;
+            if (!all_sums && cx.filter) {
+                const float thr32 = (float)G.thr64[jr];
+                const Acc32 part = pass32();
+                const float e32 = warp_sum_f(part.dE), mag = warp_sum_f(part.mag);
+                const float marg = cx.gap * mag + 1e-6f * (cx.T32 + fabsf(thr32) + fabsf(e32));
+                // (a rigid move with more terms than the sum can hold is left to the sum, which reports it)
+                const bool many = mvt != MC_MOVE_ATOM && mvt != MC_MOVE_FLIP && 3 * nq + 3 > TERM_CAP;
+                refused = !__any_sync(FULL, part.guard) && !many && e32 - thr32 > marg;
+                inter = part.cnt;
+                __syncwarp();
+            }
+            if (!refused) {
+                const int dec = exact(G.thr64[jr], nq64);
+                if (dec < 0) status = MC_ST_BOND_BREAK;
+                accept = dec == 1;
+            }
+        } else {
+            const float thr32 = G.thr32[jr];
+            const Acc32 part = pass32();
             inter = part.cnt;
             dE32 = warp_sum_f(part.dE);
             const float mag = warp_sum_f(part.mag);
@@ -1476,9 +1572,9 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
     c.h2f = ri.h2f;
     c.T64 = dy.T;
     c.T32 = dy.T32;
-    c.gap = md.recheck_gap_f;
+    c.gap = PREC == MC_PREC_FP64 ? fmaxf(md.recheck_gap_f, 1e-5f) : md.recheck_gap_f;
+    c.filter = ri.filter64 && dy.T32 > 1e-20f && dy.T32 < 1e20f;
     c.err = d.err;
-    c.pre_r2 = ri.pre_r2;
     c.r2q = ri.r2q;
     const float rconf = ri.rconf;   // (1.01 rc)^2, fixed-point units
     c.rv.smem = G.rec;
@@ -1512,7 +1608,7 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
             // evaluate attempts a .. a+nw-1, one per warp, on the same state
             const int nw = min(W, a_end - a);
             Res R;
-            if (wig < nw) R = evaluate<PREC, W>(c, G, S, G.near + wig, a + wig - a0, lane);
+            if (wig < nw) R = evaluate<PREC, W>(c, G, S, G.near + wig, a + wig - a0, lane, lg.base != nullptr);
             int adv = 1;
             if constexpr (W > 1) {
                 gsync<W>(gid);
