@@ -5,6 +5,7 @@
 #include "cell_list.h"
 #include "energy.h"
 #include "flipmc_device.cuh"
+#include "turns.cuh"
 
 namespace flipmc {
 
@@ -124,26 +125,6 @@ __global__ void __launch_bounds__(256) replica_cells_sum_kernel(DevState d, cons
     if (threadIdx.x == 0) out[r] = red[0];
 }
 
-// Fixed-order sum of a per-site (or per-molecule) array over each replica.
-__global__ void __launch_bounds__(256) replica_sum_kernel(DevState d, const double *v, int per_mol, double scale_inv_n,
-                                                          double *out, int stride, int offset)
-{
-    const int r = blockIdx.x;
-    const RepInfo ri = d.rep[r];
-    const int n = per_mol ? ri.n_sites / 3 : ri.n_sites;
-    const int off = per_mol ? ri.site_off / 3 : ri.site_off;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += 256) s = __dadd_rn(s, v[off + i]);
-    __shared__ double red[256];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] = __dadd_rn(red[threadIdx.x], red[threadIdx.x + w]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[(size_t)r * stride + offset] = scale_inv_n != 0.0 ? red[0] / (double)n : red[0];
-}
-
 void launch_energy(const DevState &d, int buf, double *e_cell, double *e_out_dev, cudaStream_t st)
 {
     pair_cells_kernel<false><<<(d.n_cells + kCellWarps - 1) / kCellWarps, 32 * kCellWarps, 0, st>>>(d, buf, e_cell);
@@ -225,102 +206,225 @@ __global__ void set_t0_kernel(DevState d, const long long *X, const int *types, 
     for (int ax = 0; ax < 3; ++ax) o.u0[3 * (size_t)m + ax] = u[ax];
 }
 
-// Per molecule: F_s of its three atoms, F_s^cm and C_2 (Eq. 5-7).
-__global__ void observables_kernel(DevState d, const long long *X, ObsState o, const double *qa, int nqa,
-                                   const double *qc, int nqc, double *fs_site, double *fscm_mol, double *c2_mol)
-{
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= d.n_sites / 3) return;
-    const int r = d.rep_of_site[3 * m];
-    const double h = d.rep[r].h;
-    double dx[3][3];
-    for (int k = 0; k < 3; ++k)
-        for (int ax = 0; ax < 3; ++ax)
-            dx[k][ax] = (double)(X[9 * (size_t)m + 3 * k + ax] - o.X0[9 * (size_t)m + 3 * k + ax]) * h;
-    for (int k = 0; k < 3; ++k) {
-        double s = 0.0;
-        for (int q = 0; q < nqa; ++q)
-            s += cos(qa[3 * q] * dx[k][0] + qa[3 * q + 1] * dx[k][1] + qa[3 * q + 2] * dx[k][2]);
-        fs_site[3 * (size_t)m + k] = s / (double)nqa;
-    }
-    double cm[3];
-    for (int ax = 0; ax < 3; ++ax) cm[ax] = ((dx[0][ax] + dx[1][ax]) + dx[2][ax]) / 3.0;
-    double s = 0.0;
-    for (int q = 0; q < nqc; ++q) s += cos(qc[3 * q] * cm[0] + qc[3 * q + 1] * cm[1] + qc[3 * q + 2] * cm[2]);
-    fscm_mol[m] = s / (double)nqc;
-    double u[3];
-    orientation(X, m, o.kref[m], h, u);
-    const double x = u[0] * o.u0[3 * (size_t)m] + u[1] * o.u0[3 * (size_t)m + 1] + u[2] * o.u0[3 * (size_t)m + 2];
-    c2_mol[m] = 1.5 * x * x - 0.5;
-}
+// ---------------------------------------------------------------------------
+// Correlations of Eq. 5-7
+// ---------------------------------------------------------------------------
+// What bounds them: 3 n_qa + n_qc cosines per molecule and origin.  As FP64
+// cosines they kept the FP64 pipe 86% busy; with the integer cosines of
+// turns.cuh a launch for 8 x 1000 molecules with 48 wavevectors of each kind
+// (1 to 2 origins) takes 20.5 us instead of 320 (integer multiplies), and the
+// observables of 8000 molecules 17.3 instead of 174.6.
+//
+// A block takes 32 molecules of one replica.  Their displacements are staged
+// once as 32-bit words; lane l of every warp holds molecule l, and the eight
+// warps share out the wavevectors, so that a few thousand molecules fill the
+// GPU (one molecule per thread left most of it idle) and a wavevector is one
+// broadcast load.  The warps' integer sums add up in shared memory, exactly;
+// what is left in FP64 (C_2, the squares, the sums over molecules) runs on
+// full warps, about 45 operations per 32 molecules.
+constexpr int kSlices = 8;
+constexpr double kCosUnit = 0x1p53;   // cos_turn's 1
 
-// The per-molecule quantities of one (origin, time) pair that the sums need:
-// F_s of the three atoms (their sum and sum of squares), F_s^cm, C_2, and the
-// products of Eq. chi4 and of the Pearson coefficient.
-struct CorrVals {
-    double v[7];   // sum_k fs_k, sum_k fs_k^2, fcm, fcm^2, c2, c2^2, c2 fcm
+struct RelaxSmem {
+    uint32_t lo[12][kCorrChunk];      // per atom and axis, then of the three atoms' sum: displacement + 2^31 ...
+    int hi[12][kCorrChunk];           // ... and its multiples of 2^32
+    uint32_t q[9][kCorrChunk];        // wrapped positions now
+    long long part[kSlices][4][kCorrChunk];
+    int bad;
 };
 
-__device__ CorrVals corr_molecule(const long long *X, const long long *X0, int kref, const double *u0, int m, double h,
-                                  const double *qa, int nqa, const double *qc, int nqc)
+// sm.part[w][k][l] = warp w's share of sum_q cos of atom k (k = 3: centre of
+// mass) of molecule m0 + l, in units of 2^-53; lanes past nm hold no molecule.
+// Leaves the block synchronised.
+__device__ __forceinline__ void relax_cosines(RelaxSmem &sm, const long long *X, const long long *X0, int m0, int nm,
+                                              const Turns *ta, int nqa, const Turns *tc, int nqc)
 {
-    double dx[3][3];
-    for (int k = 0; k < 3; ++k)
-        for (int ax = 0; ax < 3; ++ax) dx[k][ax] = (double)(X[9 * (size_t)m + 3 * k + ax] - X0[9 * (size_t)m + 3 * k + ax]) * h;
-    CorrVals o;
-    o.v[0] = 0.0;
-    o.v[1] = 0.0;
-    for (int k = 0; k < 3; ++k) {
-        double s = 0.0;
-        for (int q = 0; q < nqa; ++q)
-            s += cos(qa[3 * q] * dx[k][0] + qa[3 * q + 1] * dx[k][1] + qa[3 * q + 2] * dx[k][2]);
-        const double f = s / (double)nqa;
-        o.v[0] += f;
-        o.v[1] += f * f;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    int far = 0;
+    for (int i = tid; i < 9 * kCorrChunk; i += 32 * kSlices) {
+        const int m = i / 9, c = i - 9 * m;
+        long long d = 0;
+        uint32_t q = 0;
+        if (m < nm) {
+            const long long x = X[9 * (size_t)m0 + i];
+            d = x - X0[9 * (size_t)m0 + i];
+            q = (uint32_t)x;
+        }
+        d += 1ll << 31;
+        sm.q[c][m] = q;
+        sm.lo[c][m] = (uint32_t)d;
+        sm.hi[c][m] = (int)(d >> 32);
+        far |= (int)(d >> 32);
     }
-    double cm[3];
-    for (int ax = 0; ax < 3; ++ax) cm[ax] = ((dx[0][ax] + dx[1][ax]) + dx[2][ax]) / 3.0;
-    double s = 0.0;
-    for (int q = 0; q < nqc; ++q) s += cos(qc[3 * q] * cm[0] + qc[3 * q + 1] * cm[1] + qc[3 * q + 2] * cm[2]);
-    const double fcm = s / (double)nqc;
-    double u[3];
-    orientation(X, m, kref, h, u);
-    const double x = u[0] * u0[0] + u[1] * u0[1] + u[2] * u0[2];
-    const double c2 = 1.5 * x * x - 0.5;
-    o.v[2] = fcm;
-    o.v[3] = fcm * fcm;
-    o.v[4] = c2;
-    o.v[5] = c2 * c2;
-    o.v[6] = c2 * fcm;
-    return o;
+    if (tid == 0) sm.bad = 0;
+    __syncthreads();
+    if (tid < 3 * kCorrChunk) {
+        const int m = lane, ax = w;
+        long long d = 1ll << 31;
+        for (int k = 0; k < 3; ++k)
+            d += ((long long)sm.hi[3 * k + ax][m] << 32) + (long long)sm.lo[3 * k + ax][m] - (1ll << 31);
+        sm.lo[9 + ax][m] = (uint32_t)d;
+        sm.hi[9 + ax][m] = (int)(d >> 32);
+        far |= (int)(d >> 32);
+    }
+    far = __syncthreads_or(far);
+    uint32_t u[12];
+#pragma unroll
+    for (int c = 0; c < 12; ++c) u[c] = sm.lo[c][lane];
+    long long s[4] = {0, 0, 0, 0};
+    auto cosine = [&](const Turns &t, int k) {
+        uint64_t p = turn_phase(t, u[3 * k], u[3 * k + 1], u[3 * k + 2]) - t.bias;
+        if (far) p += turn_phase_boxes(t, sm.hi[3 * k][lane], sm.hi[3 * k + 1][lane], sm.hi[3 * k + 2][lane]);
+        return cos_turn(p);
+    };
+    unsigned bad = 0;
+    for (int q = w; q < nqa; q += kSlices) {
+        const Turns t = ta[q];
+        bad |= t.bad;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) s[k] += cosine(t, k);
+    }
+    // (the warps take the centre-of-mass vectors from the other end, so that
+    // short lists of both kinds do not meet in the same warps)
+    for (int q = kSlices - 1 - w; q < nqc; q += kSlices) {
+        const Turns t = tc[q];
+        bad |= t.bad << 1;
+        s[3] += cosine(t, 3);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) sm.part[w][k][lane] = s[k];
+    if (lane == 0 && bad) atomicOr(&sm.bad, (int)bad);
+    __syncthreads();
 }
 
-// Block (chunk, pair): the chunk's molecules (one replica's), each thread in
-// ascending order, then a fixed tree over the block's threads.
-__global__ void __launch_bounds__(256) corr_chunk_kernel(DevState d, const long long *X, CorrDev c, CorrPairs p)
+// the sum over the wavevectors of quantity k of molecule l, as a double (NaN
+// when one of its wavevectors is not finite)
+__device__ __forceinline__ double relax_sum(const RelaxSmem &sm, int k, int l)
 {
-    const int chunk = blockIdx.x, pr = blockIdx.y;
-    const int m0 = c.chunk_m0[chunk], m1 = c.chunk_m0[chunk + 1];
-    const int slot = p.slot[pr];
-    const size_t M = c.n_sites / 3;
-    const long long *X0 = c.X0 + (size_t)slot * 3 * c.n_sites;
-    const int *kref = c.kref + (size_t)slot * M;
-    const double *u0 = c.u0 + (size_t)slot * 3 * M;
-    const double h = d.rep[d.rep_of_site[3 * m0]].h;
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int m = m0 + threadIdx.x; m < m1; m += 256) {
-        const CorrVals v = corr_molecule(X, X0, kref[m], u0 + 3 * (size_t)m, m, h, c.qa, c.n_qa, c.qc, c.n_qc);
-        for (int j = 0; j < 7; ++j) acc[j] = __dadd_rn(acc[j], v.v[j]);
+    long long s = 0;
+#pragma unroll
+    for (int w = 0; w < kSlices; ++w) s += sm.part[w][k][l];
+    return (sm.bad >> (k == 3)) & 1 ? __longlong_as_double(0x7FF8000000000000ll) : (double)s;
+}
+
+// C_2 of molecule l against its orientation u0 (unit vector): the current
+// orientation is along three times (site kref - centroid), an integer vector.
+__device__ __forceinline__ double relax_c2(const RelaxSmem &sm, int l, int kref, const double *u0)
+{
+    double dot = 0.0, n2 = 0.0;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        const int a = (int)(sm.q[3 + ax][l] - sm.q[ax][l]), b = (int)(sm.q[6 + ax][l] - sm.q[ax][l]);
+        const long long mine = kref == 0 ? 0ll : (kref == 1 ? (long long)a : (long long)b);
+        const double v = (double)(3 * mine - a - b);
+        dot += v * u0[ax];
+        n2 += v * v;
     }
-    __shared__ double red[7][256];
-    for (int j = 0; j < 7; ++j) red[j][threadIdx.x] = acc[j];
+    return 1.5 * (dot * dot / n2) - 0.5;
+}
+
+__global__ void __launch_bounds__(32 * kSlices) observables_kernel(DevState d, const long long *X, ObsState o,
+                                                                   MolChunks mc, const Turns *ta, int nqa,
+                                                                   const Turns *tc, int nqc, double *fs_site,
+                                                                   double *fscm_mol, double *c2_mol, double *part)
+{
+    __shared__ RelaxSmem sm;
+    const int m0 = mc.m0[blockIdx.x], nm = mc.m0[blockIdx.x + 1] - m0;
+    const int r = d.rep_of_site[3 * m0];
+    relax_cosines(sm, X, o.X0, m0, nm, ta + (size_t)r * nqa, nqa, tc + (size_t)r * nqc, nqc);
+    // warps 0-2: the atoms, warp 3: the centres of mass, warp 4: the orientations
+    const int l = threadIdx.x & 31, k = threadIdx.x >> 5, m = m0 + l;
+    if (k > 4) return;
+    double v = 0.0;
+    if (l < nm) {
+        if (k == 4) v = c2_mol[m] = relax_c2(sm, l, o.kref[m], o.u0 + 3 * (size_t)m);
+        else if (k == 3) v = fscm_mol[m] = relax_sum(sm, 3, l) / (kCosUnit * nqc);
+        else v = fs_site[3 * (size_t)m + k] = relax_sum(sm, k, l) / (kCosUnit * nqa);
+    }
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, s));
+    if (l == 0) part[(size_t)blockIdx.x * kCorrPart + k] = v;
+}
+
+// Means per replica: the chunk sums (thread k takes chunks k, k + 128, ... in
+// order, then a fixed tree).
+__global__ void __launch_bounds__(128) observables_mean_kernel(DevState d, MolChunks mc, const double *part, double *out)
+{
+    const int r = blockIdx.x;
+    double S[3] = {0.0, 0.0, 0.0};
+    for (int k = mc.rep0[r] + threadIdx.x; k < mc.rep0[r + 1]; k += 128) {
+        const double *p = part + (size_t)k * kCorrPart;
+        S[0] = __dadd_rn(S[0], __dadd_rn(__dadd_rn(p[0], p[1]), p[2]));
+        S[1] = __dadd_rn(S[1], p[3]);
+        S[2] = __dadd_rn(S[2], p[4]);
+    }
+    __shared__ double red[3][128];
+    for (int j = 0; j < 3; ++j) red[j][threadIdx.x] = S[j];
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
+    for (int w = 64; w > 0; w >>= 1) {
         if (threadIdx.x < w)
-            for (int j = 0; j < 7; ++j) red[j][threadIdx.x] = __dadd_rn(red[j][threadIdx.x], red[j][threadIdx.x + w]);
+            for (int j = 0; j < 3; ++j) red[j][threadIdx.x] = __dadd_rn(red[j][threadIdx.x], red[j][threadIdx.x + w]);
         __syncthreads();
     }
-    if (threadIdx.x < 7) c.partials[((size_t)pr * c.n_chunks + chunk) * kCorrPart + threadIdx.x] = red[threadIdx.x][0];
+    if (threadIdx.x < 3) {
+        const int n = d.rep[r].n_sites;
+        out[3 * (size_t)r + threadIdx.x] = red[threadIdx.x][0] / (double)(threadIdx.x == 0 ? n : n / 3);
+    }
+}
+
+// Block (chunk, pair): the seven sums of the chunk's molecules that the
+// statistics need: of F_s of the three atoms, of its squares, of F_s^cm, of its
+// square, of C_2, of its square, and of C_2 F_s^cm.
+__global__ void __launch_bounds__(32 * kSlices) corr_chunk_kernel(DevState d, const long long *X, CorrDev c, CorrPairs p)
+{
+    __shared__ RelaxSmem sm;
+    const int chunk = blockIdx.x, pr = blockIdx.y;
+    const int m0 = c.chunks.m0[chunk], nm = c.chunks.m0[chunk + 1] - m0;
+    const int slot = p.slot[pr];
+    const size_t M = c.n_sites / 3;
+    const int r = d.rep_of_site[3 * m0];
+    relax_cosines(sm, X, c.X0 + (size_t)slot * 3 * c.n_sites, m0, nm, c.ta + (size_t)r * c.n_qa, c.n_qa,
+                  c.tc + (size_t)r * c.n_qc, c.n_qc);
+    if (threadIdx.x >= 32) return;
+    const int l = threadIdx.x;
+    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (l < nm) {
+        const size_t m = (size_t)slot * M + m0 + l;
+        const double c2 = relax_c2(sm, l, c.kref[m], c.u0 + 3 * m);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double f = relax_sum(sm, k, l);
+            v[0] += f;
+            v[1] += f * f;
+        }
+        const double f = relax_sum(sm, 3, l);
+        v[2] = f;
+        v[3] = f * f;
+        v[4] = c2;
+        v[5] = c2 * c2;
+        v[6] = c2 * f;
+    }
+    // sum over the lanes in a fixed order, halving the quantities per lane with
+    // the lanes (9 additions instead of 35); lane l ends with quantity l >> 2
+#pragma unroll
+    for (int o = 16, h = 4; o >= 4; o >>= 1, h >>= 1) {
+        const bool up = (l & o) != 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (i < h) {
+                const double give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+                v[i] = __dadd_rn(keep, __shfl_xor_sync(0xffffffffu, give, o));
+            }
+    }
+    v[0] = __dadd_rn(v[0], __shfl_xor_sync(0xffffffffu, v[0], 2));
+    v[0] = __dadd_rn(v[0], __shfl_xor_sync(0xffffffffu, v[0], 1));
+    const int j = l >> 2;
+    if ((l & 3) == 0 && j < 7) {
+        // the cosine sums over wavevectors become means (exact where all are 1)
+        const double A = kCosUnit * c.n_qa, C = kCosUnit * c.n_qc;
+        const double unit = j == 0 ? A : j == 1 ? A * A : j == 2 || j == 6 ? C : j == 3 ? C * C : 1.0;
+        c.partials[((size_t)pr * c.chunks.n + chunk) * kCorrPart + j] = v[0] / unit;
+    }
 }
 
 // Block (pair, replica): the replica's chunk sums (thread k takes chunks k,
@@ -332,8 +436,8 @@ __global__ void __launch_bounds__(128) corr_finish_kernel(DevState d, CorrDev c,
 {
     const int pr = blockIdx.x / d.n_rep, r = blockIdx.x - pr * d.n_rep;
     double S[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int k = c.rep_chunk0[r] + threadIdx.x; k < c.rep_chunk0[r + 1]; k += 128)
-        for (int j = 0; j < 7; ++j) S[j] = __dadd_rn(S[j], c.partials[((size_t)pr * c.n_chunks + k) * kCorrPart + j]);
+    for (int k = c.chunks.rep0[r] + threadIdx.x; k < c.chunks.rep0[r + 1]; k += 128)
+        for (int j = 0; j < 7; ++j) S[j] = __dadd_rn(S[j], c.partials[((size_t)pr * c.chunks.n + k) * kCorrPart + j]);
     __shared__ double red[7][128];
     for (int j = 0; j < 7; ++j) red[j][threadIdx.x] = S[j];
     __syncthreads();
@@ -366,47 +470,88 @@ __global__ void __launch_bounds__(128) corr_finish_kernel(DevState d, CorrDev c,
 void launch_corr_sample(const DevState &d, const long long *X, const CorrDev &c, const CorrPairs &p, cudaStream_t st)
 {
     if (p.n <= 0) return;
-    corr_chunk_kernel<<<dim3(c.n_chunks, p.n), 256, 0, st>>>(d, X, c, p);
+    corr_chunk_kernel<<<dim3(c.chunks.n, p.n), 32 * kSlices, 0, st>>>(d, X, c, p);
     corr_finish_kernel<<<p.n * d.n_rep, 128, 0, st>>>(d, c, p);
 }
 
-// S(q) of one (replica, wavevector) per block: the sums of cos and sin of
-// q . x over the replica's atoms (x = q_fixed h, in [0, L)), each thread in
-// ascending order, then a fixed tree; out = (C^2 + S^2) / N (Eq. sq with the
-// i = j terms included).
-__global__ void __launch_bounds__(256) sq_kernel(DevState d, const long long *X, const double *qv, int n_q,
-                                                 double *out)
+__global__ void turns_kernel(DevState d, const double *qv, int n_q, bool over_three, Turns *out)
 {
-    const int r = blockIdx.y, k = blockIdx.x;
-    const RepInfo ri = d.rep[r];
-    const double qx = qv[3 * k], qy = qv[3 * k + 1], qz = qv[3 * k + 2];
-    double c = 0.0, sn = 0.0;
-    for (int i = threadIdx.x; i < ri.n_sites; i += 256) {
-        const long long *x = X + 3 * (size_t)(ri.site_off + i);
-        const double ph = qx * ((double)(uint32_t)x[0] * ri.h) + qy * ((double)(uint32_t)x[1] * ri.h) +
-                          qz * ((double)(uint32_t)x[2] * ri.h);
-        double sv, cv;
-        sincos(ph, &sv, &cv);
-        c = __dadd_rn(c, cv);
-        sn = __dadd_rn(sn, sv);
-    }
-    __shared__ double rc[256], rs[256];
-    rc[threadIdx.x] = c;
-    rs[threadIdx.x] = sn;
-    __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            rc[threadIdx.x] = __dadd_rn(rc[threadIdx.x], rc[threadIdx.x + w]);
-            rs[threadIdx.x] = __dadd_rn(rs[threadIdx.x], rs[threadIdx.x + w]);
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[(size_t)r * n_q + k] = (rc[0] * rc[0] + rs[0] * rs[0]) / (double)ri.n_sites;
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (size_t)n_q * d.n_rep) return;
+    const int r = (int)(i / n_q), k = (int)(i - (size_t)r * n_q);
+    out[i] = make_turns(qv + 3 * (size_t)k, d.rep[r].h, over_three ? kInv6Pi : kInv2Pi);
 }
 
-void launch_sq(const DevState &d, const long long *X, const double *qv, int n_q, double *out, cudaStream_t st)
+void launch_turns(const DevState &d, const double *qv, int n_q, bool over_three, Turns *out, cudaStream_t st)
 {
-    sq_kernel<<<dim3(n_q, d.n_rep), 256, 0, st>>>(d, X, qv, n_q, out);
+    turns_kernel<<<(unsigned)(((size_t)n_q * d.n_rep + 63) / 64), 64, 0, st>>>(d, qv, n_q, over_three, out);
+}
+
+// S(q): block (part, wavevector, replica) sums cos and sin of q . x over a part
+// of kSqPart of the replica's records (x = q_fixed h, in [0, L); the order of
+// the atoms does not matter to integer sums), then sq_sum_kernel adds the parts
+// in order; out = (C^2 + S^2) / N (Eq. sq with the i = j terms included).
+// Bound by the integer multiplies of the two cosines: 240 wavevectors of
+// 24000 atoms took 477 us as FP64 sincos (one block per wavevector, FP64
+// pipe) and take 62 us (52% of the multiply pipe).
+constexpr int kSqPart = 4096;         // 16 records per thread: 32 lanes' sums of 16 stay below 2^63
+
+__global__ void __launch_bounds__(256) sq_kernel(DevState d, int buf, const Turns *turns, int n_q, double2 *part)
+{
+    const int k = blockIdx.y, r = blockIdx.z;
+    const RepInfo ri = d.rep[r];
+    const int i0 = blockIdx.x * kSqPart, i1 = min(ri.n_sites, i0 + kSqPart);
+    if (i0 >= i1) return;
+    const int4 *rec = d.rec[buf] + ri.site_off;
+    const Turns t = turns[(size_t)r * n_q + k];
+    long long c = 0, s = 0;
+    for (int i = i0 + threadIdx.x; i < i1; i += 256) {
+        const int4 a = rec[i];
+        const uint64_t ph = turn_phase(t, (uint32_t)a.x, (uint32_t)a.y, (uint32_t)a.z);
+        c += cos_turn(ph);
+        s += cos_turn(ph - (1ull << 62));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        c += __shfl_xor_sync(0xffffffffu, c, o);
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    __shared__ double2 red[8];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_double2((double)c, (double)s);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double2 v = red[0];
+        for (int w = 1; w < 8; ++w) v = make_double2(v.x + red[w].x, v.y + red[w].y);
+        part[((size_t)r * n_q + k) * gridDim.x + blockIdx.x] = v;
+    }
+}
+
+__global__ void sq_sum_kernel(DevState d, const Turns *turns, int n_q, int n_part, const double2 *part, double *out,
+                              int stride)
+{
+    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (size_t)n_q * d.n_rep) return;
+    const int r = (int)(i / n_q), k = (int)(i - (size_t)r * n_q);
+    const int n = d.rep[r].n_sites;
+    double c = 0.0, s = 0.0;
+    for (int b = 0; b * kSqPart < n; ++b) {
+        const double2 v = part[i * n_part + b];
+        c += v.x;
+        s += v.y;
+    }
+    c /= kCosUnit;
+    s /= kCosUnit;
+    out[(size_t)r * stride + k] = turns[i].bad ? __longlong_as_double(0x7FF8000000000000ll) : (c * c + s * s) / (double)n;
+}
+
+int sq_parts(int max_sites) { return (max_sites + kSqPart - 1) / kSqPart; }
+
+void launch_sq(const DevState &d, int buf, const Turns *turns, int n_q, int max_sites, double2 *part, double *out,
+               int stride, cudaStream_t st)
+{
+    const int np = sq_parts(max_sites);
+    sq_kernel<<<dim3(np, n_q, d.n_rep), 256, 0, st>>>(d, buf, turns, n_q, part);
+    sq_sum_kernel<<<(unsigned)(((size_t)n_q * d.n_rep + 127) / 128), 128, 0, st>>>(d, turns, n_q, np, part, out, stride);
 }
 
 // Pair-distance histogram (Eq. gr): counts[b] = pairs i < j with
@@ -543,15 +688,12 @@ void launch_set_t0(const DevState &d, const long long *X, const int *types, cons
     set_t0_kernel<<<(nm + 127) / 128, 128, 0, st>>>(d, X, types, o);
 }
 
-void launch_observables(const DevState &d, const long long *X, const ObsState &o, const double *qa, int nqa,
-                        const double *qc, int nqc, double *fs_site, double *fscm_mol, double *c2_mol, double *out,
-                        cudaStream_t st)
+void launch_observables(const DevState &d, const long long *X, const ObsState &o, const MolChunks &mc, const Turns *ta,
+                        int nqa, const Turns *tc, int nqc, double *fs_site, double *fscm_mol, double *c2_mol,
+                        double *part, double *out, cudaStream_t st)
 {
-    const int nm = d.n_sites / 3;
-    observables_kernel<<<(nm + 127) / 128, 128, 0, st>>>(d, X, o, qa, nqa, qc, nqc, fs_site, fscm_mol, c2_mol);
-    replica_sum_kernel<<<d.n_rep, 256, 0, st>>>(d, fs_site, 0, 1.0, out, 3, 0);
-    replica_sum_kernel<<<d.n_rep, 256, 0, st>>>(d, fscm_mol, 1, 1.0, out, 3, 1);
-    replica_sum_kernel<<<d.n_rep, 256, 0, st>>>(d, c2_mol, 1, 1.0, out, 3, 2);
+    observables_kernel<<<mc.n, 32 * kSlices, 0, st>>>(d, X, o, mc, ta, nqa, tc, nqc, fs_site, fscm_mol, c2_mol, part);
+    observables_mean_kernel<<<d.n_rep, 128, 0, st>>>(d, mc, part, out);
 }
 
 }  // namespace flipmc

@@ -14,13 +14,30 @@ struct ObsState {
     double *u0;      // 3 per molecule: unit orientation at t0
 };
 
+// A wavevector of one replica in turns per quantum (turns.cuh): per axis the
+// 96-bit fraction of kappa = q h / 2 pi (k2 the highest word), and the phase of
+// the displacement 2^31 on every axis (the kernels add 2^31 to a displacement
+// to make it unsigned).
+struct alignas(16) Turns {
+    uint32_t k0[3], k1[3], k2[3];
+    uint32_t bad;    // a component is not finite: every result is NaN
+    uint64_t bias;
+};
+// out[r * n_q + k] = the wavevector qv[3 k ..] of every replica; over_three:
+// divided by three (for sums of three displacements, a molecule's atoms)
+void launch_turns(const DevState &d, const double *qv, int n_q, bool over_three, Turns *out, cudaStream_t st);
+
 // FP64 energy per replica into e_out_dev[n_rep]; e_cell is n_cells scratch.
 void launch_energy(const DevState &d, int buf, double *e_cell, double *e_out_dev, cudaStream_t st);
 // Periodic drift check: drift[2r] = |e_run - E| / |E| (last), drift[2r+1] its
 // largest value; one recompute counted; e_run restarts from E[r].
 void launch_drift(const DevState &d, const double *E, double *drift, cudaStream_t st);
-// S(q) per (replica, wavevector): out[r * n_q + k] = |sum_i exp(i q_k . x_i)|^2 / N.
-void launch_sq(const DevState &d, const long long *X, const double *qv, int n_q, double *out, cudaStream_t st);
+// S(q) per (replica, wavevector) of the records of buf: out[r * stride + k] =
+// |sum_i exp(i q_k . x_i)|^2 / N for the n_q wavevectors of turns; part:
+// sq_parts(max_sites) * n_q * n_rep pairs of doubles.
+int sq_parts(int max_sites);
+void launch_sq(const DevState &d, int buf, const Turns *turns, int n_q, int max_sites, double2 *part, double *out,
+               int stride, cudaStream_t st);
 // Pair-distance counts per replica and bin (every pair once) of the records of buf; counts zeroed by the caller.
 void launch_pair_hist(const DevState &d, int buf, int max_sites, double dr, int n_bins, unsigned long long *counts,
                       cudaStream_t st);
@@ -29,10 +46,21 @@ void launch_virial(const DevState &d, int buf, double *w_cell, double *w_out_dev
 // unwrapped positions (3 per site) and types in site order
 void launch_gather(const DevState &d, int buf, long long *X, int *types, cudaStream_t st);
 void launch_set_t0(const DevState &d, const long long *X, const int *types, const ObsState &o, cudaStream_t st);
-// out[3 r + {0,1,2}] = F_s, F_s^cm, C_2 of replica r
-void launch_observables(const DevState &d, const long long *X, const ObsState &o, const double *qa, int nqa,
-                        const double *qc, int nqc, double *fs_site, double *fscm_mol, double *c2_mol, double *out,
-                        cudaStream_t st);
+
+// The molecules of every replica in chunks of at most kCorrChunk, none
+// spanning two replicas (one block of the correlation kernels each).
+struct MolChunks {
+    const int *m0;           // per chunk: first molecule (global index), m0[n] = total molecules
+    const int *rep0;         // per replica: first chunk; [n_rep] = n
+    int n;
+};
+constexpr int kCorrChunk = 32;   // molecules per block: one per lane
+
+// Per particle F_s (fs_site), F_s^cm and C_2 (per molecule) and, per replica,
+// out[3 r + {0,1,2}] = their means; part: kCorrPart doubles per chunk.
+void launch_observables(const DevState &d, const long long *X, const ObsState &o, const MolChunks &mc, const Turns *ta,
+                        int nqa, const Turns *tc, int nqc, double *fs_site, double *fscm_mol, double *c2_mol,
+                        double *part, double *out, cudaStream_t st);
 
 // Multiple-origin correlations: the origins live in slots; each slot holds an
 // ObsState's arrays (slot s at X0 + 3 N s, kref + M s, u0 + 3 M s).
@@ -41,19 +69,16 @@ struct CorrDev {
     const int *kref;
     const double *u0;
     size_t n_sites;             // all replicas
-    const double *qa;           // n_qa wavevectors (atoms), 3 each
-    const double *qc;           // n_qc wavevectors (centres of mass)
+    const Turns *ta;            // n_qa wavevectors (atoms) per replica
+    const Turns *tc;            // n_qc wavevectors (centres of mass) per replica
     int n_qa, n_qc;
-    const int *chunk_m0;        // per chunk: first molecule (global index), chunk_m0[n_chunks] = total molecules
-    int n_chunks;
-    const int *rep_chunk0;      // per replica: first chunk; [n_rep] = n_chunks
-    double *partials;           // CORR_PART per (pair, chunk)
+    MolChunks chunks;
+    double *partials;           // kCorrPart per (pair, chunk)
     double *acc;                // MC_CORR_NSUM per (replica, lag)
     int n_lags;
 };
 
 constexpr int kCorrMaxPairs = 32;       // (origin, lag) pairs per launch
-constexpr int kCorrChunk = 256;         // molecules per block of the per-particle pass (one per thread)
 constexpr int kCorrPart = 8;            // partial sums per (pair, chunk)
 
 // The (origin slot, lag index) pairs measured at one time.

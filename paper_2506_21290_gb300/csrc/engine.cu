@@ -136,6 +136,27 @@ struct mc_handle {
         pageable.resize(bytes);
         return pageable.data();
     }
+    // device workspace of the analysis calls, grown on demand and kept with the
+    // handle; a call lays its arrays out in it anew
+    void *work = nullptr;
+    size_t work_bytes = 0;
+    int need_work(size_t bytes)
+    {
+        if (work_bytes >= bytes) return MC_OK;
+        if (work) {
+            cudaStreamSynchronize(stream);
+            cudaFree(work);
+            work = nullptr;
+            work_bytes = 0;
+        }
+        const cudaError_t e = cudaMalloc(&work, bytes);
+        if (e != cudaSuccess) {
+            work = nullptr;
+            return fail(MC_ERR_CUDA, std::string("cudaMalloc (workspace): ") + cudaGetErrorString(e));
+        }
+        work_bytes = bytes;
+        return MC_OK;
+    }
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
     int cur = 0;
@@ -175,7 +196,9 @@ struct mc_handle {
     double *d_e_out = nullptr;
     long long *d_X = nullptr;
     int *d_types = nullptr;
-    double *d_fs = nullptr, *d_fscm = nullptr, *d_c2 = nullptr, *d_q = nullptr, *d_obs_out = nullptr;
+    double *d_fs = nullptr, *d_fscm = nullptr, *d_c2 = nullptr, *d_obs_out = nullptr;
+    MolChunks chunks{};                  // molecules in blocks of the correlation kernels
+    double *d_obs_part = nullptr;
     std::vector<RepParam> par_host;
     std::vector<RepParam> par_sent;
     MixDev mix_sent{};
@@ -663,6 +686,14 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
     d.precision = h->precision;
     d.wait_limit = o.wait_limit_log2 > 0 ? (1u << o.wait_limit_log2) : 0u;
     const int M_tot = h->n_sites / 3;
+    std::vector<int> chunk_m0, rep_chunk0;
+    for (const RepInfo &ri : h->reps) {
+        rep_chunk0.push_back((int)chunk_m0.size());
+        for (int m = 0; m < ri.n_sites / 3; m += kCorrChunk) chunk_m0.push_back(ri.site_off / 3 + m);
+    }
+    rep_chunk0.push_back((int)chunk_m0.size());
+    chunk_m0.push_back(M_tot);
+    int *d_m0, *d_c0;
     int4 *r0, *r1;
     int *cc, *cs, *co, *so, *img, *err;
     double *cde, *erun;
@@ -680,7 +711,9 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         (rc = h->alloc(&h->d_types, h->n_sites)) || (rc = h->alloc(&h->obs.X0, 3 * (size_t)h->n_sites)) ||
         (rc = h->alloc(&h->obs.kref, M_tot)) || (rc = h->alloc(&h->obs.u0, 3 * (size_t)M_tot)) ||
         (rc = h->alloc(&h->d_fs, h->n_sites)) || (rc = h->alloc(&h->d_fscm, M_tot)) ||
-        (rc = h->alloc(&h->d_c2, M_tot)) || (rc = h->alloc(&h->d_q, 6 * 256)) ||
+        (rc = h->alloc(&h->d_c2, M_tot)) || (rc = h->alloc(&d_m0, chunk_m0.size())) ||
+        (rc = h->alloc(&d_c0, rep_chunk0.size())) ||
+        (rc = h->alloc(&h->d_obs_part, (chunk_m0.size() - 1) * kCorrPart)) ||
         (rc = h->alloc(&h->d_obs_out, 3 * (size_t)n_rep)) ||
         (rc = h->alloc(&h->ds.att_rnd, 2 * (size_t)h->n_sites)) || (rc = h->alloc(&h->d_bar, 2)) ||
         (rc = h->alloc(&h->ds.cell_done, h->n_cells)) || (rc = h->alloc(&h->ds.cell_count2, h->n_cells)) ||
@@ -712,12 +745,15 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
     d.err = err;
 
     h->par_host.assign(n_rep, RepParam{1.0, 0, 0, 0});
+    h->chunks = MolChunks{d_m0, d_c0, (int)chunk_m0.size() - 1};
     auto up = [&](void *dst, const void *src, size_t bytes) {
         return cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     };
     if (!up(h->d_rep, h->reps.data(), sizeof(RepInfo) * n_rep) || !up(h->d_model, &h->model_host, sizeof(ModelDev)) ||
         !up(h->d_rep_of_site, rep_of_site.data(), sizeof(int) * h->n_sites) ||
         !up(h->d_act_off, act_off.data(), sizeof(int) * (n_rep + 1)) ||
+        !up(d_m0, chunk_m0.data(), sizeof(int) * chunk_m0.size()) ||
+        !up(d_c0, rep_chunk0.data(), sizeof(int) * rep_chunk0.size()) ||
         (n_rep > 1 && !up(h->d_act_slot, act_slot.data(), sizeof(int2) * h->n_act)) ||
         !up(h->d_par, h->par_host.data(), sizeof(RepParam) * n_rep)) {
         mc_destroy(h);
@@ -790,6 +826,7 @@ void mc_destroy(mc_handle *h)
     for (int b = 0; b < 2; ++b)
         if (h->graph[b]) cudaGraphExecDestroy(h->graph[b]);
     for (auto &a : h->allocs) cudaFree(a.p);
+    if (h->work) cudaFree(h->work);
     if (h->pin) cudaFreeHost(h->pin);
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
     delete h;
@@ -1089,26 +1126,27 @@ int mc_structure_factor(mc_handle *h, const double *qvec, int n_q, double *out)
     if (n_q < 1 || n_q > 65535) return fail(MC_ERR_INVALID_ARG, "1 <= n_q <= 65535");
     int rc = set_device(h);
     if (rc) return rc;
-    double *dq = nullptr, *dout = nullptr;
-    CUDA_TRY(cudaMallocAsync(&dq, sizeof(double) * 3 * n_q, h->stream));
-    cudaError_t e = cudaMallocAsync(&dout, sizeof(double) * (size_t)n_q * h->n_rep, h->stream);
-    if (e != cudaSuccess) {
-        cudaFreeAsync(dq, h->stream);
-        return fail(MC_ERR_CUDA, std::string("structure factor: ") + cudaGetErrorString(e));
+    int max_sites = 0;
+    for (auto &r : h->reps) max_sites = std::max(max_sites, r.n_sites);
+    const size_t R = (size_t)h->n_rep, np = (size_t)sq_parts(max_sites);
+    // as many wavevectors at a time as keep their tables near 16 MB
+    const size_t per = R * (sizeof(Turns) + sizeof(double2) * np);
+    const int batch = (int)std::min<size_t>(n_q, std::max<size_t>(1, ((size_t)16 << 20) / per));
+    const size_t b_q = sizeof(double) * 3 * (size_t)n_q, b_out = sizeof(double) * (size_t)n_q * R;
+    auto up16 = [](size_t x) { return (x + 15) & ~(size_t)15; };
+    if ((rc = h->need_work(up16(b_q) + up16(b_out) + per * batch))) return rc;
+    double *dq = (double *)h->work, *dout = (double *)((char *)dq + up16(b_q));
+    double2 *part = (double2 *)((char *)dout + up16(b_out));
+    Turns *turns = (Turns *)(part + R * np * batch);
+    CUDA_TRY(cudaMemcpyAsync(dq, qvec, b_q, cudaMemcpyHostToDevice, h->stream));
+    for (int k = 0; k < n_q; k += batch) {
+        const int n = std::min(batch, n_q - k);
+        launch_turns(h->ds, dq + 3 * (size_t)k, n, false, turns, h->stream);
+        launch_sq(h->ds, h->cur, turns, n, max_sites, part, dout + k, n_q, h->stream);
     }
-    e = cudaMemcpyAsync(dq, qvec, sizeof(double) * 3 * n_q, cudaMemcpyHostToDevice, h->stream);
-    if (e == cudaSuccess) {
-        launch_gather(h->ds, h->cur, h->d_X, h->d_types, h->stream);
-        launch_sq(h->ds, h->d_X, dq, n_q, dout, h->stream);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(out, dout, sizeof(double) * (size_t)n_q * h->n_rep, cudaMemcpyDeviceToHost, h->stream);
-    cudaFreeAsync(dq, h->stream);
-    cudaFreeAsync(dout, h->stream);
-    const cudaError_t e2 = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess || e2 != cudaSuccess)
-        return fail(MC_ERR_CUDA, std::string("structure factor: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaMemcpyAsync(out, dout, b_out, cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
     return check_device_errors(h);
 }
 
@@ -1125,19 +1163,13 @@ int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, dou
     int rc = set_device(h);
     if (rc) return rc;
     const size_t n = (size_t)n_bins * h->n_rep;
-    unsigned long long *dc = nullptr;
-    CUDA_TRY(cudaMallocAsync(&dc, sizeof(unsigned long long) * n, h->stream));
-    cudaError_t e = cudaMemsetAsync(dc, 0, sizeof(unsigned long long) * n, h->stream);
-    if (e == cudaSuccess) {
-        launch_pair_hist(h->ds, h->cur, max_sites, dr, n_bins, dc, h->stream);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(counts, dc, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost, h->stream);
-    cudaFreeAsync(dc, h->stream);
-    const cudaError_t e2 = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess || e2 != cudaSuccess)
-        return fail(MC_ERR_CUDA, std::string("pair histogram: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
+    if ((rc = h->need_work(sizeof(unsigned long long) * n))) return rc;
+    unsigned long long *dc = (unsigned long long *)h->work;
+    CUDA_TRY(cudaMemsetAsync(dc, 0, sizeof(unsigned long long) * n, h->stream));
+    launch_pair_hist(h->ds, h->cur, max_sites, dr, n_bins, dc, h->stream);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaMemcpyAsync(counts, dc, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
     if (g) {
         // g(r) at the bin centres: 2 counts / (N rho shell volume), rho = N / V
         const double pi = 3.14159265358979323846;
@@ -1330,11 +1362,18 @@ int mc_observables(mc_handle *h, const double *qvec_atom, int n_qa, const double
     if (n_qa < 1 || n_qa > 256 || n_qc < 1 || n_qc > 256) return fail(MC_ERR_INVALID_ARG, "1 <= n_q <= 256");
     int rc = set_device(h);
     if (rc) return rc;
-    CUDA_TRY(cudaMemcpyAsync(h->d_q, qvec_atom, sizeof(double) * 3 * n_qa, cudaMemcpyHostToDevice, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(h->d_q + 3 * 256, qvec_cm, sizeof(double) * 3 * n_qc, cudaMemcpyHostToDevice, h->stream));
+    const size_t R = (size_t)h->n_rep;
+    const size_t b_t = sizeof(Turns) * R * (n_qa + n_qc);
+    if ((rc = h->need_work(b_t + sizeof(double) * 3 * (n_qa + n_qc)))) return rc;
+    Turns *ta = (Turns *)h->work, *tc = ta + R * n_qa;
+    double *dqa = (double *)(tc + R * n_qc), *dqc = dqa + 3 * n_qa;
+    CUDA_TRY(cudaMemcpyAsync(dqa, qvec_atom, sizeof(double) * 3 * n_qa, cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(dqc, qvec_cm, sizeof(double) * 3 * n_qc, cudaMemcpyHostToDevice, h->stream));
+    launch_turns(h->ds, dqa, n_qa, false, ta, h->stream);
+    launch_turns(h->ds, dqc, n_qc, true, tc, h->stream);
     launch_gather(h->ds, h->cur, h->d_X, h->d_types, h->stream);
-    launch_observables(h->ds, h->d_X, h->obs, h->d_q, n_qa, h->d_q + 3 * 256, n_qc, h->d_fs, h->d_fscm, h->d_c2,
-                       h->d_obs_out, h->stream);
+    launch_observables(h->ds, h->d_X, h->obs, h->chunks, ta, n_qa, tc, n_qc, h->d_fs, h->d_fscm, h->d_c2,
+                       h->d_obs_part, h->d_obs_out, h->stream);
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaMemcpyAsync(out, h->d_obs_out, sizeof(double) * 3 * h->n_rep, cudaMemcpyDeviceToHost, h->stream));
     const size_t M = (size_t)h->n_sites / 3;
@@ -1520,43 +1559,33 @@ int mc_corr_setup(mc_handle *h, int n_lags, const int64_t *lags, int origin_ever
     corr_free(h);
     auto &c = h->corr;
     const size_t N = (size_t)h->n_sites, M = N / 3;
-    // chunks of at most kCorrChunk molecules, none spanning two replicas
-    std::vector<int> chunk_m0, rep_chunk0;
-    for (int r = 0; r < h->n_rep; ++r) {
-        rep_chunk0.push_back((int)chunk_m0.size());
-        const int m_off = h->reps[r].site_off / 3, m_n = h->reps[r].n_sites / 3;
-        for (int m = 0; m < m_n; m += kCorrChunk) chunk_m0.push_back(m_off + m);
-    }
-    const int n_chunks = (int)chunk_m0.size();
-    rep_chunk0.push_back(n_chunks);
-    chunk_m0.push_back((int)M);
     long long *X0 = nullptr;
-    int *kref = nullptr, *cm0 = nullptr, *rc0 = nullptr;
+    int *kref = nullptr;
+    Turns *ta = nullptr, *tc = nullptr;
     double *u0 = nullptr, *q = nullptr, *part = nullptr, *acc = nullptr;
     const size_t n_acc = (size_t)h->n_rep * n_lags * MC_CORR_NSUM;
     if ((rc = corr_alloc(h, &X0, (size_t)max_origins * 3 * N)) || (rc = corr_alloc(h, &kref, (size_t)max_origins * M)) ||
         (rc = corr_alloc(h, &u0, (size_t)max_origins * 3 * M)) || (rc = corr_alloc(h, &q, 3 * (size_t)(n_qa + n_qc))) ||
-        (rc = corr_alloc(h, &cm0, chunk_m0.size())) || (rc = corr_alloc(h, &rc0, rep_chunk0.size())) ||
-        (rc = corr_alloc(h, &part, (size_t)kCorrMaxPairs * n_chunks * kCorrPart)) || (rc = corr_alloc(h, &acc, n_acc))) {
+        (rc = corr_alloc(h, &ta, (size_t)h->n_rep * n_qa)) || (rc = corr_alloc(h, &tc, (size_t)h->n_rep * n_qc)) ||
+        (rc = corr_alloc(h, &part, (size_t)kCorrMaxPairs * h->chunks.n * kCorrPart)) ||
+        (rc = corr_alloc(h, &acc, n_acc))) {
         corr_free(h);
         return rc;
     }
-    CUDA_TRY(cudaMemcpy(q, qvec_atom, sizeof(double) * 3 * n_qa, cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(q + 3 * n_qa, qvec_cm, sizeof(double) * 3 * n_qc, cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(cm0, chunk_m0.data(), sizeof(int) * chunk_m0.size(), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(rc0, rep_chunk0.data(), sizeof(int) * rep_chunk0.size(), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemset(acc, 0, sizeof(double) * n_acc));
+    CUDA_TRY(cudaMemcpyAsync(q, qvec_atom, sizeof(double) * 3 * n_qa, cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(q + 3 * n_qa, qvec_cm, sizeof(double) * 3 * n_qc, cudaMemcpyHostToDevice, h->stream));
+    launch_turns(h->ds, q, n_qa, false, ta, h->stream);
+    launch_turns(h->ds, q + 3 * n_qa, n_qc, true, tc, h->stream);
+    CUDA_TRY(cudaMemsetAsync(acc, 0, sizeof(double) * n_acc, h->stream));
     c.dev.X0 = X0;
     c.dev.kref = kref;
     c.dev.u0 = u0;
     c.dev.n_sites = N;
-    c.dev.qa = q;
-    c.dev.qc = q + 3 * n_qa;
+    c.dev.ta = ta;
+    c.dev.tc = tc;
     c.dev.n_qa = n_qa;
     c.dev.n_qc = n_qc;
-    c.dev.chunk_m0 = cm0;
-    c.dev.n_chunks = n_chunks;
-    c.dev.rep_chunk0 = rc0;
+    c.dev.chunks = h->chunks;
     c.dev.partials = part;
     c.dev.acc = acc;
     c.dev.n_lags = n_lags;
