@@ -155,12 +155,9 @@ __global__ void cl_order_kernel(DevState d, int buf)
     if (c < d.n_cells) cl_order_cells4(d, buf, c, lane);
 }
 
-void launch_cell_list(const DevState &d, int buf_in, int buf_out, cudaStream_t st)
+void launch_cell_sort(const DevState &d, int buf_in, int buf_out, cudaStream_t st)
 {
     const int tb = 256;
-    const int nb = (d.n_sites + tb - 1) / tb;
-    cudaMemsetAsync(d.cell_count, 0, sizeof(int) * d.n_cells, st);
-    cl_count_kernel<<<nb, tb, 0, st>>>(d, buf_in);
     if (d.scan_part != nullptr && d.n_cells > 8 * kScanCells) {
         const int nb = (d.n_cells + kScanCells - 1) / kScanCells;
         cl_scan_part_kernel<<<nb, 256, 0, st>>>(d);
@@ -169,9 +166,17 @@ void launch_cell_list(const DevState &d, int buf_in, int buf_out, cudaStream_t s
     } else {
         cl_scan_kernel<<<1, 1024, 0, st>>>(d);
     }
-    cl_scatter_kernel<<<nb, tb, 0, st>>>(d, buf_in, buf_out);
+    cl_scatter_kernel<<<(d.n_sites + tb - 1) / tb, tb, 0, st>>>(d, buf_in, buf_out);
     const int wpb = 8;
     cl_order_kernel<<<(d.n_cells + 4 * wpb - 1) / (4 * wpb), 32 * wpb, 0, st>>>(d, buf_out);
+}
+
+void launch_cell_list(const DevState &d, int buf_in, int buf_out, cudaStream_t st)
+{
+    const int tb = 256;
+    cudaMemsetAsync(d.cell_count, 0, sizeof(int) * d.n_cells, st);
+    cl_count_kernel<<<(d.n_sites + tb - 1) / tb, tb, 0, st>>>(d, buf_in);
+    launch_cell_sort(d, buf_in, buf_out, st);
 }
 
 }  // namespace flipmc

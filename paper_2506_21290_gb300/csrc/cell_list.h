@@ -14,6 +14,8 @@ __global__ void cl_order_kernel(DevState d, int buf);
 
 // count + scan + scatter + per-cell ordering: records of buf_in, cell-sorted into buf_out.
 void launch_cell_list(const DevState &d, int buf_in, int buf_out, cudaStream_t st);
+// the same from counts already taken (scan + scatter + ordering)
+void launch_cell_sort(const DevState &d, int buf_in, int buf_out, cudaStream_t st);
 
 // Attempt-log destination of a logged sweep (null base: no log).
 struct LogArgs {

@@ -5,130 +5,139 @@
 #include "cell_list.h"
 #include "energy.h"
 #include "flipmc_device.cuh"
+#include "pair_walk.cuh"
 #include "turns.cuh"
 
 namespace flipmc {
 
-// Energy (VIRIAL = false) or pair virial (VIRIAL = true), one warp per cell:
-// every pair (i, j) with i an atom of the cell and j an atom of the 27 (or,
-// for n_c = 2, the 8) neighbour cells with a larger site index.  Lane k walks
-// neighbour cell k; pairs of different molecules beyond every cutoff (FP32
-// screen with a 1% margin) add exactly 0 and are dropped; the others are
-// gathered in order into a ring and evaluated in FP64 32 at a time, one per
-// lane, so the FP64 pipe works on full warps.  Each lane sums its pairs in
-// gathering order and a fixed butterfly adds the lanes: the cell's sum is the
-// same on every run for a given state.
-constexpr int kCellWarps = 8;       // cells per block
-constexpr int kRing = 64;           // gathered pairs per warp (at most 63 waiting)
+// ln y to about two units, y in (0, 1]: the atanh series of ln_series with
+// fused steps and the walk's reciprocal.  NaN below 0, -inf at 0.
+__device__ __forceinline__ double walk_ln(double y)
+{
+    const long long bits = __double_as_longlong(y);
+    int e = (int)((bits >> 52) & 0x7FF) - 1023;
+    double m = __longlong_as_double((bits & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
+    if (m > 0x1.6a09e667f3bcdp+0) {
+        m *= 0.5;
+        e += 1;
+    }
+    const double z = (m - 1.0) * walk_rcp(m + 1.0), w = z * z;
+    double s = 2.0 / 23.0;
+    s = fma(s, w, 2.0 / 21.0);
+    s = fma(s, w, 2.0 / 19.0);
+    s = fma(s, w, 2.0 / 17.0);
+    s = fma(s, w, 2.0 / 15.0);
+    s = fma(s, w, 2.0 / 13.0);
+    s = fma(s, w, 2.0 / 11.0);
+    s = fma(s, w, 2.0 / 9.0);
+    s = fma(s, w, 2.0 / 7.0);
+    s = fma(s, w, 2.0 / 5.0);
+    s = fma(s, w, 2.0 / 3.0);
+    s = fma(s, w, 2.0);
+    const double r = fma((double)e, 0x1.62e42fefa39efp-1, z * s);
+    return y > 0.0 ? r : (y == 0.0 ? -__longlong_as_double(0x7FF0000000000000ll) : __longlong_as_double(0x7FF8000000000000ll));
+}
+
+// Energy (VIRIAL = false) or pair virial (VIRIAL = true) of every replica: each
+// pair from its atom of the smaller site index (pair_walk.cuh), FP64.  A warp
+// walks one to four cells and keeps what does not fill a batch of 32 pairs for
+// the next; bonds, whose Eq. 2 costs three times Eq. 1, wait in a ring of their
+// own for full batches.  The sums (per lane, then lanes, warps and blocks) run in
+// a fixed order: the same on every run for a given state.
+// Energy of 24000 atoms 41 us (62 with the sum over cells, when every lane of a
+// warp walked a neighbour cell and bonds shared the batches), of 192000 atoms
+// 133 (290), of 256 replicas with 823000 atoms 505 (1161).
+template <bool VIRIAL>
+struct EnergyWalk {
+    const ModelDev &md;
+    const Quantum2 hh;
+    const double c24;
+    const int4 *ring;
+    double *bond_r2;               // [64] waiting bonds, and their type pairs
+    int *bond_ab;
+    const int lane;
+    int bond_head = 0, bond_tail = 0;
+    double acc = 0.0;
+
+    __device__ void own(int, int, const int4 &) {}
+    __device__ void atom(int, int) {}
+    __device__ void part(int, int) {}
+    __device__ void done() {}
+    __device__ void eval(int at, int n)
+    {
+        const bool on = lane < n;
+        const int4 e = ring[(at + (on ? lane : 0)) & (kWalkRing - 1)];
+        const int ab = walk_types(e.w);
+        const double r2 = walk_r2(e, hh);
+        const double t = md.s2[ab] * walk_rcp(r2);
+        const double s6 = t * t * t;
+        const double v = VIRIAL ? c24 * (s6 * fma(2.0, s6, -1.0)) : fma(md.e4 * s6, s6 - 1.0, md.eps);
+        if (on && r2 < md.rc2[ab]) acc += v;
+        const bool bond = on && walk_bonded(e.w);
+        const unsigned b = __ballot_sync(0xffffffffu, bond);
+        if (bond) {
+            const int k = (bond_tail + __popc(b & ((1u << lane) - 1u))) & 63;
+            bond_r2[k] = r2;
+            bond_ab[k] = ab;
+        }
+        bond_tail += __popc(b);
+        if (bond_tail - bond_head >= 32) bonds(32);
+    }
+    __device__ void bonds(int n)
+    {
+        __syncwarp();
+        if (lane < n) {
+            const int k = (bond_head + lane) & 63;
+            const double x = bond_r2[k] * md.invR2[bond_ab[k]];
+            acc += VIRIAL ? 2.0 * md.nke * x * walk_rcp(1.0 - x) : md.nke * walk_ln(1.0 - x);
+        }
+        bond_head += n;
+        __syncwarp();
+    }
+};
 
 template <bool VIRIAL>
-__global__ void __launch_bounds__(32 * kCellWarps) pair_cells_kernel(DevState d, int buf, double *e_cell)
+__global__ void __launch_bounds__(32 * kEnergyWarps) pair_energy_kernel(DevState d, int buf, double *part, double *out)
 {
-    __shared__ int2 ring_all[kCellWarps][kRing];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int c = blockIdx.x * kCellWarps + wib;
-    if (c >= d.n_cells) return;   // the whole warp
-    int2 *ring = ring_all[wib];
-    const int s0 = d.cell_start[c];
-    const int n = d.cell_start[c + 1] - s0;
-    double acc = 0.0;
-    if (n > 0) {
-        const int r = d.rep_of_site[s0];
-        const RepInfo ri = d.rep[r];
-        const ModelDev &md = *d.model;
-        const int4 *rec = d.rec[buf];
-        const int nc = ri.nc, cl = c - ri.cell_off;
-        const int cx = cl % nc, cy = (cl / nc) % nc, cz = cl / (nc * nc);
-        const bool small = nc == 2;
-        const int ns = small ? 8 : 27;
-        int cst = 0, cnt = 0;
-        if (lane < ns) {
-            int ox, oy, oz;
-            if (small) {
-                ox = lane & 1; oy = (lane >> 1) & 1; oz = lane >> 2;
-            } else {
-                ox = lane % 3 - 1; oy = (lane / 3) % 3 - 1; oz = lane / 9 - 1;
-            }
-            const int nb = ri.cell_off + (((cz + oz + nc) % nc) * nc + (cy + oy + nc) % nc) * nc + (cx + ox + nc) % nc;
-            cst = d.cell_start[nb];
-            cnt = d.cell_start[nb + 1] - cst;
-        }
-        const int maxc = __reduce_max_sync(0xffffffffu, cnt);
-        float rc2max = 0.f;
-        for (int k = 0; k < 9; ++k) rc2max = fmaxf(rc2max, md.rc2f[k]);
-        const float pre = rc2max * 1.01f;
-        const unsigned lt = (1u << lane) - 1u;
-        int head = 0, tail = 0;   // warp-uniform
-        auto eval = [&](int e) {
-            const int2 p = ring[e & (kRing - 1)];
-            const int4 me = rec[s0 + p.x], o = rec[p.y];
-            const int dx = (int)((uint32_t)o.x - (uint32_t)me.x);
-            const int dy = (int)((uint32_t)o.y - (uint32_t)me.y);
-            const int dz = (int)((uint32_t)o.z - (uint32_t)me.z);
-            const double r2 = r2_fixed64(dx, dy, dz, ri.h);
-            const bool bonded = rec_mol(o.w) == rec_mol(me.w);
-            const int ab = 3 * rec_type(me.w) + rec_type(o.w);
-            acc = __dadd_rn(acc, VIRIAL ? virial64(md, r2, ab, bonded) : phi64(md, r2, ab, bonded));
-        };
-        for (int i = 0; i < n; ++i) {
-            const int4 me = rec[s0 + i];
-            const int si = rec_site(me.w), mi = rec_mol(me.w);
-            for (int k = 0; k < maxc; ++k) {
-                bool hit = false;
-                if (k < cnt) {
-                    const int4 o = rec[cst + k];
-                    if (rec_site(o.w) > si) {
-                        if (rec_mol(o.w) == mi) {
-                            hit = true;
-                        } else {
-                            const float fx = (float)(int)((uint32_t)o.x - (uint32_t)me.x) * ri.hf;
-                            const float fy = (float)(int)((uint32_t)o.y - (uint32_t)me.y) * ri.hf;
-                            const float fz = (float)(int)((uint32_t)o.z - (uint32_t)me.z) * ri.hf;
-                            hit = fx * fx + fy * fy + fz * fz <= pre;
-                        }
-                    }
-                }
-                const unsigned b = __ballot_sync(0xffffffffu, hit);
-                if (hit) ring[(tail + __popc(b & lt)) & (kRing - 1)] = make_int2(i, cst + k);
-                tail += __popc(b);
-                if (tail - head >= 32) {
-                    __syncwarp();
-                    eval(head + lane);
-                    head += 32;
-                    __syncwarp();
-                }
-            }
-        }
-        __syncwarp();
-        if (lane < tail - head) eval(head + lane);
+    __shared__ WalkSmem walk[kEnergyWarps];
+    __shared__ double bond_r2[kEnergyWarps][64], red[32 * kEnergyWarps];
+    __shared__ int bond_ab[kEnergyWarps][64];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int r = 0, c0 = 0, b0 = 0;
+    if (d.cells.unit != nullptr) {
+        const int2 u = d.cells.unit[blockIdx.x];
+        r = u.x;
+        c0 = u.y;
+        b0 = d.cells.rep0[r];
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc = __dadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, o));
-    if (lane == 0) e_cell[c] = acc;
-}
-
-// Fixed-order sum of the per-cell values of each replica (one block each).
-__global__ void __launch_bounds__(256) replica_cells_sum_kernel(DevState d, const double *v, double *out)
-{
-    const int r = blockIdx.x;
     const RepInfo ri = d.rep[r];
-    const int n = ri.nc * ri.nc * ri.nc;
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += 256) s = __dadd_rn(s, v[ri.cell_off + i]);
-    __shared__ double red[256];
-    red[threadIdx.x] = s;
+    const int n_cells = ri.nc * ri.nc * ri.nc, per = walk_cells(ri.n_sites, n_cells);
+    if (d.cells.unit == nullptr) c0 = blockIdx.x * kEnergyWarps * per;
+    const ModelDev &md = *d.model;
+    EnergyWalk<VIRIAL> p{md, quantum2(ri.h), 6.0 * md.e4, walk[w].ring, bond_r2[w], bond_ab[w], lane};
+    int head = 0, tail = 0;
+    for (int k = 0; k < per; ++k)
+        walk_cell<true>(d, ri, md, d.rec[buf], c0 + w * per + k, lane, walk[w], head, tail, p);
+    if (tail > head) p.eval(head, tail - head);
+    if (p.bond_tail > p.bond_head) p.bonds(p.bond_tail - p.bond_head);
+    double v = p.acc;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0) red[w] = v;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] = __dadd_rn(red[threadIdx.x], red[threadIdx.x + w]);
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < kEnergyWarps; ++k) v = __dadd_rn(v, red[k]);
+        part[blockIdx.x] = v;
     }
-    if (threadIdx.x == 0) out[r] = red[0];
+    const int nb = n_cells / (kEnergyWarps * per);
+    if (!last_block(d.arrived + r, nb)) return;
+    v = sum_parts<32 * kEnergyWarps>(part + b0, nb, red);
+    if (threadIdx.x == 0) out[r] = v;
 }
 
-void launch_energy(const DevState &d, int buf, double *e_cell, double *e_out_dev, cudaStream_t st)
+void launch_energy(const DevState &d, int buf, double *part, double *e_out_dev, cudaStream_t st)
 {
-    pair_cells_kernel<false><<<(d.n_cells + kCellWarps - 1) / kCellWarps, 32 * kCellWarps, 0, st>>>(d, buf, e_cell);
-    replica_cells_sum_kernel<<<d.n_rep, 256, 0, st>>>(d, e_cell, e_out_dev);
+    pair_energy_kernel<false><<<d.cells.n, 32 * kEnergyWarps, 0, st>>>(d, buf, part, e_out_dev);
 }
 
 // Drift check of the running total against a fresh FP64 recompute E, per
@@ -152,10 +161,9 @@ void launch_drift(const DevState &d, const double *E, double *drift, cudaStream_
     drift_kernel<<<(d.n_rep + 127) / 128, 128, 0, st>>>(d, E, drift);
 }
 
-void launch_virial(const DevState &d, int buf, double *w_cell, double *w_out_dev, cudaStream_t st)
+void launch_virial(const DevState &d, int buf, double *part, double *w_out_dev, cudaStream_t st)
 {
-    pair_cells_kernel<true><<<(d.n_cells + kCellWarps - 1) / kCellWarps, 32 * kCellWarps, 0, st>>>(d, buf, w_cell);
-    replica_cells_sum_kernel<<<d.n_rep, 256, 0, st>>>(d, w_cell, w_out_dev);
+    pair_energy_kernel<true><<<d.cells.n, 32 * kEnergyWarps, 0, st>>>(d, buf, part, w_out_dev);
 }
 
 // Unwrapped fixed-point positions and types in site-index order.

@@ -24,6 +24,7 @@
 #include "energy.h"
 #include "flipmc_types.h"
 #include "md.h"
+#include "pair_walk.cuh"
 
 using namespace flipmc;
 
@@ -180,7 +181,7 @@ struct mc_handle {
         MdDev dev{};
         std::vector<double> T, Q;
         std::vector<void *> bufs;
-        cudaGraphExec_t graph[2] = {nullptr, nullptr};
+        cudaGraphExec_t graph[2][2] = {};   // one step and kMdGraphSteps, from either buffer
     } md;
     std::vector<Buf> allocs;
     // device scratch
@@ -257,7 +258,8 @@ void build_model(const mc_params &p, double gap, ModelDev &md)
             md.s2f[ab] = (float)md.s2[ab];
             md.rc2f[ab] = (float)md.rc2[ab];
             md.R2f[ab] = (float)md.R2[ab];
-            md.invR2f[ab] = (float)(1.0 / md.R2[ab]);
+            md.invR2[ab] = 1.0 / md.R2[ab];
+            md.invR2f[ab] = (float)md.invR2[ab];
         }
     md.eps = p.eps;
     md.e4 = 4.0 * p.eps;
@@ -281,6 +283,26 @@ bool fp32_bound_holds(const ModelDev &md, double L)
     bool ok = normal(md.eps) && (md.ke == 0.0 || normal(md.ke)) && L > 1e-6 && L < 1e6;
     for (int k = 0; k < 9; ++k) ok = ok && normal(md.s2[k]) && normal(md.R2[k]);
     return ok;
+}
+
+// Work units over the replicas: `range` gives a replica's {first, count} and how
+// many go to a unit.
+struct HostUnits {
+    std::vector<int2> unit;
+    std::vector<int> rep0;
+};
+
+template <class F>
+HostUnits make_units(const std::vector<RepInfo> &reps, const F &range)
+{
+    HostUnits u;
+    for (size_t r = 0; r < reps.size(); ++r) {
+        u.rep0.push_back((int)u.unit.size());
+        const auto [ext, per] = range(reps[r]);
+        for (int k = 0; k < ext.second; k += per) u.unit.push_back(make_int2((int)r, ext.first + k));
+    }
+    u.rep0.push_back((int)u.unit.size());
+    return u;
 }
 
 // Longest interaction range: the WCA cutoff of any type pair, and the FENE
@@ -693,6 +715,12 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
     }
     rep_chunk0.push_back((int)chunk_m0.size());
     chunk_m0.push_back(M_tot);
+    const HostUnits cell_units = make_units(h->reps, [](const RepInfo &ri) {
+        const int n = ri.nc * ri.nc * ri.nc;
+        return std::make_pair(std::make_pair(ri.cell_off, n), kEnergyWarps * walk_cells(ri.n_sites, n));
+    });
+    int2 *d_cells;
+    int *d_cells0;
     int *d_m0, *d_c0;
     int4 *r0, *r1;
     int *cc, *cs, *co, *so, *img, *err;
@@ -713,6 +741,8 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         (rc = h->alloc(&h->d_fs, h->n_sites)) || (rc = h->alloc(&h->d_fscm, M_tot)) ||
         (rc = h->alloc(&h->d_c2, M_tot)) || (rc = h->alloc(&d_m0, chunk_m0.size())) ||
         (rc = h->alloc(&d_c0, rep_chunk0.size())) ||
+        (rc = h->alloc(&d_cells, cell_units.unit.size())) || (rc = h->alloc(&d_cells0, cell_units.rep0.size())) ||
+        (rc = h->alloc(&d.arrived, n_rep)) ||
         (rc = h->alloc(&h->d_obs_part, (chunk_m0.size() - 1) * kCorrPart)) ||
         (rc = h->alloc(&h->d_obs_out, 3 * (size_t)n_rep)) ||
         (rc = h->alloc(&h->ds.att_rnd, 2 * (size_t)h->n_sites)) || (rc = h->alloc(&h->d_bar, 2)) ||
@@ -746,6 +776,7 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
 
     h->par_host.assign(n_rep, RepParam{1.0, 0, 0, 0});
     h->chunks = MolChunks{d_m0, d_c0, (int)chunk_m0.size() - 1};
+    d.cells = Units{d_cells, d_cells0, (int)cell_units.unit.size()};
     auto up = [&](void *dst, const void *src, size_t bytes) {
         return cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     };
@@ -754,6 +785,8 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         !up(h->d_act_off, act_off.data(), sizeof(int) * (n_rep + 1)) ||
         !up(d_m0, chunk_m0.data(), sizeof(int) * chunk_m0.size()) ||
         !up(d_c0, rep_chunk0.data(), sizeof(int) * rep_chunk0.size()) ||
+        !up(d_cells, cell_units.unit.data(), sizeof(int2) * cell_units.unit.size()) ||
+        !up(d_cells0, cell_units.rep0.data(), sizeof(int) * cell_units.rep0.size()) ||
         (n_rep > 1 && !up(h->d_act_slot, act_slot.data(), sizeof(int2) * h->n_act)) ||
         !up(h->d_par, h->par_host.data(), sizeof(RepParam) * n_rep)) {
         mc_destroy(h);
@@ -810,8 +843,9 @@ static void corr_free(mc_handle *h)
 static void md_free(mc_handle *h)
 {
     if (h->stream) cudaStreamSynchronize(h->stream);
-    for (int b = 0; b < 2; ++b)
-        if (h->md.graph[b]) cudaGraphExecDestroy(h->md.graph[b]);
+    for (auto &g : h->md.graph)
+        for (int b = 0; b < 2; ++b)
+            if (g[b]) cudaGraphExecDestroy(g[b]);
     for (void *b : h->md.bufs) cudaFree(b);
     h->md = mc_handle::Md{};
 }
@@ -1740,26 +1774,29 @@ DevState md_state(const mc_handle *h)
     return d;
 }
 
-// One MD step from the records of buf (the cell-sorted current buffer) into buf ^ 1, as a graph.
-int md_graph(mc_handle *h, int buf)
+// Steps of the larger MD graph (even, so that it ends in the buffer it began
+// with): between two graph launches the GPU idles for a few microseconds, which
+// is a good part of a small system's step: 50 steps of 1000 molecules 2.04 ms with
+// one step per graph, 1.89 with eight.
+constexpr int kMdGraphSteps = 8;
+
+// MD steps as a graph, from the records of buf (the cell-sorted current buffer):
+// one, into buf ^ 1, or kMdGraphSteps.
+int md_graph(mc_handle *h, bool many, int buf)
 {
-    if (h->md.graph[buf]) return MC_OK;
+    if (h->md.graph[many][buf]) return MC_OK;
     cudaStream_t cs;
     CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t g;
     CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     const DevState d = md_state(h);
-    launch_md_begin(d, h->md.dev, cs);
-    launch_md_drift(d, buf, h->md.dev, cs);
-    launch_cell_list(d, buf, buf ^ 1, cs);
-    launch_md_forces(d, buf ^ 1, h->md.dev, cs);
-    launch_md_end(d, h->md.dev, cs);
+    for (int k = 0; k < (many ? kMdGraphSteps : 1); ++k) launch_md_step(d, buf ^ (k & 1), h->md.dev, cs);
     cudaError_t e = cudaStreamEndCapture(cs, &g);
     if (e != cudaSuccess) {
         cudaStreamDestroy(cs);
         return fail(MC_ERR_CUDA, std::string("MD graph capture: ") + cudaGetErrorString(e));
     }
-    e = cudaGraphInstantiate(&h->md.graph[buf], g, 0);
+    e = cudaGraphInstantiate(&h->md.graph[many][buf], g, 0);
     cudaGraphDestroy(g);
     cudaStreamDestroy(cs);
     if (e != cudaSuccess) return fail(MC_ERR_CUDA, std::string("MD graph instantiate: ") + cudaGetErrorString(e));
@@ -1787,55 +1824,52 @@ int mc_md_setup(mc_handle *h, double dt, double tau_T, const double *T, const do
     m.Q.resize(h->n_rep);
     for (int r = 0; r < h->n_rep; ++r)   // tau_T <= 0: no thermostat (Q infinite, xi stays 0)
         m.Q[r] = tau_T > 0.0 ? 3.0 * h->reps[r].n_sites * T[r] * tau_T * tau_T : HUGE_VAL;
-    // chunks of at most kMdChunk atoms, none spanning two replicas
-    std::vector<int> chunk_a0, rep_chunk0;
-    for (int r = 0; r < h->n_rep; ++r) {
-        rep_chunk0.push_back((int)chunk_a0.size());
-        for (int a = 0; a < h->reps[r].n_sites; a += kMdChunk) chunk_a0.push_back(h->reps[r].site_off + a);
-    }
-    const int n_chunks = (int)chunk_a0.size();
-    rep_chunk0.push_back(n_chunks);
-    chunk_a0.push_back((int)N);
     const size_t R = (size_t)h->n_rep;
-    double *bufs[9] = {};
-    const size_t sizes[9] = {3 * N, 3 * N, R, R, R, R, R, R, (size_t)n_chunks};
-    int *ibufs[2] = {};
-    const size_t isizes[2] = {chunk_a0.size(), rep_chunk0.size()};
-    for (int k = 0; k < 11; ++k) {
+    const bool fp32 = force_precision == MC_PREC_FP32;
+    const HostUnits units = make_units(h->reps, [&](const RepInfo &ri) {
+        return fp32 ? std::make_pair(std::make_pair(ri.site_off, ri.n_sites), 32)
+                    : std::make_pair(std::make_pair(ri.cell_off, ri.nc * ri.nc * ri.nc), kMdWarps);
+    });
+    const size_t nu = units.unit.size();
+    double *bufs[10] = {};
+    const size_t sizes[12] = {3 * N, 3 * N, R, R, R, R, R, R, R, nu, nu, R + 1};
+    int2 *d_unit = nullptr;
+    int *d_unit0 = nullptr;
+    for (int k = 0; k < 12; ++k) {
         void *p = nullptr;
-        const size_t bytes = k < 9 ? sizeof(double) * sizes[k] : sizeof(int) * isizes[k - 9];
+        const size_t bytes = sizes[k] * (k < 10 ? sizeof(double) : k == 10 ? sizeof(int2) : sizeof(int));
         cudaError_t e = cudaMalloc(&p, bytes);
         if (e != cudaSuccess) {
             md_free(h);
             return fail(MC_ERR_CUDA, std::string("cudaMalloc (MD): ") + cudaGetErrorString(e));
         }
         m.bufs.push_back(p);
-        CUDA_TRY(cudaMemset(p, 0, bytes));
-        if (k < 9) bufs[k] = (double *)p;
-        else ibufs[k - 9] = (int *)p;
+        CUDA_TRY(cudaMemsetAsync(p, 0, bytes, h->stream));
+        if (k < 10) bufs[k] = (double *)p;
+        else if (k == 10) d_unit = (int2 *)p;
+        else d_unit0 = (int *)p;
     }
     m.dev.v = bufs[0];
     m.dev.F = bufs[1];
     m.dev.xi = bufs[2];
     m.dev.eta = bufs[3];
-    m.dev.K = bufs[4];
-    m.dev.T = bufs[5];
-    m.dev.Q = bufs[6];
-    m.dev.scale = bufs[7];
-    m.dev.part = bufs[8];
-    m.dev.chunk_a0 = ibufs[0];
-    m.dev.rep_chunk0 = ibufs[1];
-    m.dev.n_chunks = n_chunks;
-    m.dev.fp32_forces = force_precision == MC_PREC_FP32 ? 1 : 0;
+    m.dev.xi_mid = bufs[4];
+    m.dev.eta_mid = bufs[5];
+    m.dev.scale = bufs[6];
+    m.dev.T = bufs[7];
+    m.dev.Q = bufs[8];
+    m.dev.part = bufs[9];
+    m.dev.units = Units{d_unit, d_unit0, (int)nu};
+    m.dev.fp32_forces = fp32;
     m.dev.dt = dt;
     m.dev.hdt = 0.5 * dt;
-    CUDA_TRY(cudaMemcpy(ibufs[0], chunk_a0.data(), sizeof(int) * chunk_a0.size(), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(ibufs[1], rep_chunk0.data(), sizeof(int) * rep_chunk0.size(), cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(bufs[0], v0, sizeof(double) * 3 * N, cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(bufs[5], m.T.data(), sizeof(double) * h->n_rep, cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(bufs[6], m.Q.data(), sizeof(double) * h->n_rep, cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpyAsync(d_unit, units.unit.data(), sizeof(int2) * nu, cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(d_unit0, units.rep0.data(), sizeof(int) * (R + 1), cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(bufs[0], v0, sizeof(double) * 3 * N, cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(bufs[7], m.T.data(), sizeof(double) * R, cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(cudaMemcpyAsync(bufs[8], m.Q.data(), sizeof(double) * R, cudaMemcpyHostToDevice, h->stream));
     // the forces of the current state (its cell list is current)
-    launch_md_forces(md_state(h), h->cur, m.dev, h->stream);
+    launch_md_setup(md_state(h), h->cur, m.dev, h->stream);
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     m.on = true;
@@ -1849,10 +1883,14 @@ int mc_md_run(mc_handle *h, int n_steps)
     if (n_steps < 0) return fail(MC_ERR_INVALID_ARG, "n_steps < 0");
     int rc = set_device(h);
     if (rc) return rc;
-    for (int s = 0; s < n_steps; ++s) {
-        if ((rc = md_graph(h, h->cur))) return rc;
-        CUDA_TRY(cudaGraphLaunch(h->md.graph[h->cur], h->stream));
-        h->cur ^= 1;
+    // each step counts into cell_count and leaves it zero for the next
+    if (n_steps > 0) CUDA_TRY(cudaMemsetAsync(h->ds.cell_count, 0, sizeof(int) * h->n_cells, h->stream));
+    for (int s = 0; s < n_steps;) {
+        const bool many = n_steps - s >= kMdGraphSteps;
+        if ((rc = md_graph(h, many, h->cur))) return rc;
+        CUDA_TRY(cudaGraphLaunch(h->md.graph[many][h->cur], h->stream));
+        if (!many) h->cur ^= 1;
+        s += many ? kMdGraphSteps : 1;
     }
     // the running energy of later MC sweeps starts from the MD configuration
     if (n_steps > 0) {

@@ -13,6 +13,7 @@ struct ModelDev {
     double rc2[9];   // (2^(1/3)) sigma_ab^2: WCA cutoff squared
     double R2[9];    // (R0 sigma_ab)^2: FENE divergence squared
     double eps, e4, nke, ke;
+    double invR2[9];
     float s2f[9], rc2f[9], R2f[9], invR2f[9];
     float epsf, e4f, nkef, kef;
     float bond_guard_f;   // FP32 bond-length ratio beyond which FP32 defers to FP64
@@ -78,11 +79,23 @@ enum {
     STAT_N = 16
 };
 
+// warps per block of the energy walk and of the FP64 forces (a replica has a
+// multiple of eight cells, so a block's cells are one replica's)
+constexpr int kEnergyWarps = 2;
+constexpr int kMdWarps = 4;
+
 // error bits
 enum {
     ERR_STENCIL = 1,    // neighbourhood larger than the staging capacity
     ERR_TERMS = 2,      // FP64 ordered-sum buffer overflow
     ERR_TIMEOUT = 4,
+};
+
+// Work units of a walk over all replicas, none spanning two (null tables: one replica).
+struct Units {
+    const int2 *unit;    // per unit: {replica, first cell or record}
+    const int *rep0;     // per replica: first unit; [n_rep] = n
+    int n;
 };
 
 // Everything a kernel needs, by value.
@@ -100,6 +113,8 @@ struct DevState {
     const ModelDev *model;
     const MixDev *mix;
     const int *rep_of_site;
+    Units cells;         // blocks of kEnergyWarps x walk_cells cells (energy walks; pair_walk.cuh)
+    unsigned *arrived;   // per replica: blocks of a walk that have written their sum (zero between launches)
     const int *act_off;  // n_rep + 1 prefix of (nc/2)^3
     const int2 *act_slot;    // per active-cell slot of a colour (n_act), in schedule order: {replica, active
                              // cell within the replica}; null for one replica (slot = active cell)

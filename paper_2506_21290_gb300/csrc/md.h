@@ -13,30 +13,23 @@ namespace flipmc {
 struct MdDev {
     double *v;         // 3 per site
     double *F;         // 3 per site
-    double *xi;        // per replica: thermostat friction
+    double *xi;        // per replica: thermostat friction at the end of the last step
     double *eta;       // per replica: its time integral (for the conserved energy)
-    double *K;         // per replica: kinetic energy at the last thermostat step
+    double *xi_mid;    // per replica: both after the first thermostat half step of the next step,
+    double *eta_mid;   //              which follows from the same kinetic energy
+    double *scale;     // per replica: exp(-xi_mid dt/2)
     const double *T;   // per replica: bath temperature
     const double *Q;   // per replica: thermostat mass g T tau^2, g = 3 N
-    double *scale;     // per replica: exp(-xi dt/2) of the current xi
-    double *part;      // per chunk: partial kinetic energy
-    const int *chunk_a0;     // per chunk: first atom (global); [n_chunks] = all atoms
-    const int *rep_chunk0;   // per replica: first chunk; [n_rep] = n_chunks
-    int n_chunks;
+    Units units;       // blocks of the force kernel: kMdWarps cells (FP64), or 32 records (FP32)
+    double *part;      // per block: partial sum of v^2
     int fp32_forces;   // 1: pair forces in FP32 (velocities, positions and thermostat stay FP64)
     double dt;
     double hdt;        // dt / 2
 };
 
-constexpr int kMdChunk = 2048;   // atoms per block of the kinetic-energy partial sums
-
-// Thermostat half step, then the scaling and the first half kick (start of a step).
-void launch_md_begin(const DevState &d, const MdDev &m, cudaStream_t st);
-// Positions q += rint(v dt / h) on the records of buf (cell-sorted), periodic images counted.
-void launch_md_drift(const DevState &d, int buf, const MdDev &m, cudaStream_t st);
-// Forces on every atom from its partners in the 27 (or 8) neighbour cells of buf (FP64, or FP32 pair terms).
-void launch_md_forces(const DevState &d, int buf, const MdDev &m, cudaStream_t st);
-// Second half kick, the scaling, then the thermostat half step (end of a step).
-void launch_md_end(const DevState &d, const MdDev &m, cudaStream_t st);
+// The forces of the current state and the first thermostat half step of the first step.
+void launch_md_setup(const DevState &d, int buf, const MdDev &m, cudaStream_t st);
+// One step from the cell-sorted records of buf into buf ^ 1.  cell_count must be zero, and is again afterwards.
+void launch_md_step(const DevState &d, int buf, const MdDev &m, cudaStream_t st);
 
 }  // namespace flipmc

@@ -29,6 +29,7 @@
 #include "cell_list.h"
 #include "energy.h"
 #include "flipmc_types.h"
+#include "pair_walk.cuh"
 
 using namespace flipmc;
 
@@ -48,7 +49,8 @@ constexpr size_t kOffModel = al256(kOffCtr + sizeof(RepCtr));
 constexpr size_t kOffMix = al256(kOffModel + sizeof(ModelDev));
 constexpr size_t kOffActOff = al256(kOffMix + sizeof(MixDev));
 constexpr size_t kOffErr = al256(kOffActOff + 2 * sizeof(int));
-constexpr size_t kOffRepOfSite = al256(kOffErr + sizeof(int));
+constexpr size_t kOffArrived = al256(kOffErr + sizeof(int));
+constexpr size_t kOffRepOfSite = al256(kOffArrived + sizeof(unsigned));
 constexpr size_t kOffRec0 = al256(kOffRepOfSite + sizeof(int) * kMaxSites);
 constexpr size_t kOffRec1 = al256(kOffRec0 + sizeof(int4) * kMaxSites);
 constexpr size_t kOffCount = al256(kOffRec1 + sizeof(int4) * kMaxSites);
@@ -57,7 +59,6 @@ constexpr size_t kOffCellOf = al256(kOffStart + sizeof(int) * (kMaxCells + 1));
 constexpr size_t kOffSlotOf = al256(kOffCellOf + sizeof(int) * kMaxSites);
 constexpr size_t kOffESite = al256(kOffSlotOf + sizeof(int) * kMaxSites);
 constexpr size_t kScratchBytes = al256(kOffESite + sizeof(double) * kMaxSites);
-static_assert(kMaxCells <= kMaxSites, "the partial-sum region holds one double per cell");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -108,6 +109,7 @@ __global__ void noalloc_init_kernel(Header hd, unsigned char *base, int n_sites)
         ((int *)(base + kOffActOff))[0] = hd.act_off[0];
         ((int *)(base + kOffActOff))[1] = hd.act_off[1];
         *(int *)(base + kOffErr) = 0;
+        *(unsigned *)(base + kOffArrived) = 0;
     }
     int *rep_of_site = (int *)(base + kOffRepOfSite);
     for (int i = threadIdx.x; i < n_sites; i += blockDim.x) rep_of_site[i] = 0;
@@ -193,7 +195,8 @@ extern "C" int mc_energy_noalloc(double L, int n_mol, const uint32_t *dev_q, con
             hd.model.s2f[ab] = (float)hd.model.s2[ab];
             hd.model.rc2f[ab] = (float)hd.model.rc2[ab];
             hd.model.R2f[ab] = (float)hd.model.R2[ab];
-            hd.model.invR2f[ab] = (float)(1.0 / hd.model.R2[ab]);
+            hd.model.invR2[ab] = 1.0 / hd.model.R2[ab];
+            hd.model.invR2f[ab] = (float)hd.model.invR2[ab];
         }
     hd.model.eps = p.eps;
     hd.model.e4 = 4.0 * p.eps;
@@ -222,7 +225,9 @@ extern "C" int mc_energy_noalloc(double L, int n_mol, const uint32_t *dev_q, con
     d.cell_start = (int *)(base + kOffStart);
     d.cell_of = (int *)(base + kOffCellOf);
     d.slot_of = (int *)(base + kOffSlotOf);
-    double *e_part = (double *)(base + kOffESite);   // per-cell partial sums
+    d.arrived = (unsigned *)(base + kOffArrived);
+    d.cells.n = n_cells / (kEnergyWarps * walk_cells(n_sites, n_cells));
+    double *e_part = (double *)(base + kOffESite);   // per-block partial sums
 
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t x) {
