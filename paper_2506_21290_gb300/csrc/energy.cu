@@ -570,8 +570,8 @@ void launch_sq(const DevState &d, int buf, const Turns *turns, int n_q, int max_
 // of a pipe that does 2 per SM and cycle; a pass over the 2.9e8 pairs of 8000
 // molecules took 20.4 ms.  Here the bin comes from FP32 arithmetic on the
 // exact int32 differences, and FP64 decides only the pairs that FP32 cannot
-// place for certain: 0.44 ms for the same pass, bound by instruction issue (69%
-// of the slots, 42 instructions a pair).
+// place for certain: 0.36 ms for the same pass, bound by instruction issue (36
+// instructions a pair).
 //
 // The FP32 value of f = r / dr is within 6.5 units of 2^-24 of its own size
 // (each difference rounds once when converted, three products and sums,
@@ -641,16 +641,13 @@ __global__ void __launch_bounds__(kHistTile) pair_hist_kernel(DevState d, int bu
         if (tid < nj) tile[tid] = rec[j0 + tid];
         __syncthreads();
         const int4 me = rec[min(i, N - 1)];
-        // the first partner: every j of another tile, the later ones of its own
-        const int first = i >= N ? nj : (dist == 0 ? tid + 1 : 0);
-#pragma unroll 4
-        for (int j = 0; j < nj; ++j) {
-            const int4 o = tile[j];
+        // one pair: place it, and count it when its bin is one of the histogram's
+        auto place = [&](const int4 &o, bool on) {
             const int dx = (int)((uint32_t)o.x - (uint32_t)me.x), dy = (int)((uint32_t)o.y - (uint32_t)me.y),
                       dz = (int)((uint32_t)o.z - (uint32_t)me.z);
             const float fx = (float)dx, fy = (float)dy, fz = (float)dz;
-            float root;
-            asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(fmaf(fx, fx, fmaf(fy, fy, fz * fz))));
+            float root;   // (of a sum of integer squares: 0 or at least 1)
+            asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(root) : "f"(fmaf(fx, fx, fmaf(fy, fy, fz * fz))));
             // bin = round(f - 1/2) by the exponent trick: 1.5 x 2^23 + g rounds
             // g to an integer, which then stands in the low bits (for g of
             // 2^22 and more, a value that exceeds every n_bins)
@@ -658,11 +655,18 @@ __global__ void __launch_bounds__(kHistTile) pair_hist_kernel(DevState d, int bu
             const float t = g + 12582912.0f;
             const float off = g - (t - 12582912.0f);
             int bin = __float_as_int(t) - 0x4B400000;
-            if (j >= first && bin <= n_bins) {
-                if (fabsf(off) > fmaf(-6e-7f, g, 0.499999f))
-                    bin = pair_bin64(dx, dy, dz, ri.h, ri.inv_h, dr, off > 0.f ? bin + 1 : bin);
-                if (bin < n_bins) atomicAdd(mine + (bin << SH), 1u);
-            }
+            const bool near = on && bin <= n_bins;   // (the last edge may be this pair's)
+            if (near && fabsf(off) > fmaf(-6e-7f, g, 0.499999f))
+                bin = pair_bin64(dx, dy, dz, ri.h, ri.inv_h, dr, off > 0.f ? bin + 1 : bin);
+            if (near && bin < n_bins) atomicAdd(mine + (bin << SH), 1u);
+        };
+        if (dist == 0) {
+            for (int j = 0; j < nj; ++j) place(tile[j], j > tid && i < N);
+        } else if (nj == kHistTile && (ti + 1) * kHistTile <= N) {
+#pragma unroll 4
+            for (int j = 0; j < kHistTile; ++j) place(tile[j], true);
+        } else {
+            for (int j = 0; j < nj; ++j) place(tile[j], i < N);
         }
         // a 32-bit count takes at most 2^17 tile pairs of 2^14 pairs
         if (++done == 1u << 17) {
