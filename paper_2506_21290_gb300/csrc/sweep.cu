@@ -1210,7 +1210,7 @@ __device__ __forceinline__ bool clashes(const Near *near, int wb, float rconf, i
 {
     const Near &B = near[wb];
     bool hit = false;
-#pragma unroll
+#pragma unroll 1
     for (int wa = 0; wa < W - 1; ++wa) {
         const Near &A = near[wa];
         const bool live = (wa < wb) && A.accept != 0;
@@ -1240,7 +1240,11 @@ __device__ __forceinline__ unsigned tally_inc(const Res &R, int lane)
     return inc;
 }
 
-// Apply attempt R (number `at` in the cell) to the staged state and log it.
+// Apply attempt R (number `at` in the cell) to the staged state and to the
+// cell's records in global memory, and log it.  (A cell changes about one record
+// in two phases: writing those when they change leaves the end of a phase no
+// stores to wait for before it publishes the cell: 256 replicas 826 -> 801 us a
+// sweep, 64000 molecules 248.1 -> 245.5, 1000 molecules 64.1 -> 63.1.)
 // One thread (lane 0 of the warp that evaluated it).  A moved atom whose
 // fixed-point coordinate wraps around the box counts the periodic image it
 // enters (img, per global site): only the cell that owns the atom moves it,
@@ -1248,7 +1252,7 @@ __device__ __forceinline__ unsigned tally_inc(const Res &R, int lane)
 // the cell's net displacement.
 template <int PREC>
 __device__ __forceinline__ void commit(const Group &G, const Res &R, int at, const LogArgs &lg, const RepInfo &ri,
-                                       uint64_t sweep, int own_start, int *img)
+                                       uint64_t sweep, int own_start, int *img, int4 *own)
 {
     if (R.accept) {
         if (R.mvt == MC_MOVE_FLIP) {
@@ -1256,7 +1260,7 @@ __device__ __forceinline__ void commit(const Group &G, const Res &R, int at, con
             for (int s = 0; s < 2; ++s) {
                 int4 rs = G.rec[R.ks[s]];
                 rs.w = (rs.w & ~3) | R.t3n[s];
-                G.rec[R.ks[s]] = rs;
+                G.rec[R.ks[s]] = own[R.ks[s]] = rs;
             }
         } else {
 #pragma unroll
@@ -1275,7 +1279,7 @@ __device__ __forceinline__ void commit(const Group &G, const Res &R, int at, con
                     rs.x = (int)R.qn[s][0];
                     rs.y = (int)R.qn[s][1];
                     rs.z = (int)R.qn[s][2];
-                    G.rec[ks] = rs;
+                    G.rec[ks] = own[ks] = rs;
                 }
             }
         }
@@ -1355,11 +1359,83 @@ __device__ __forceinline__ void signal_done(unsigned int *done)
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(done) : "memory");
 }
 
+// What a multi-warp group of a persistent launch with one cell per colour keeps
+// of its eight cells, so that a phase does not fetch it anew: between the
+// neighbours' last phase and the group's next one, the replica's parameters, the
+// extents of the cells and the draws were three dependent trips to L2 (the polls
+// of the wait drop the first-level cache), about 1900 of a phase's 11000 cycles;
+// now the draws, from a known place, are under way while the group polls.
+// The eight cells and all their neighbours are 4 x 4 x 4 cells.  A sweep of 8000
+// molecules 77.3 -> 74.6 us, of 8 x 1000 80.8 -> 77.8, of 1000 63.1 -> 61.7.  (A
+// kernel with both ways in it spilled 140 bytes: 88.9 us; hence the template.)
+struct CellCache {
+    RepInfo ri;
+    RepParam par;
+    uint32_t shift[3];
+    int r, ax, ay, az;           // replica, and the cell block 2a .. 2a + 1 per axis
+    int4 ext[64];                // {first record, records, cell}: cells 2a - 1 .. 2a + 2 per axis, x fastest
+};
+
+struct Draws {
+    uint4 b0, b1;                // attempt `lane`'s draws (warp 0)
+    double t64;
+    float t32;
+};
+
+template <int PREC>
+__device__ __forceinline__ void load_draws(const DevState &d, int start, int n, int lane, Draws &w)
+{
+    if (lane < n) {
+        const size_t slot = (size_t)start + (size_t)lane;
+        w.b0 = d.att_rnd[2 * slot];
+        w.b1 = d.att_rnd[2 * slot + 1];
+        if (PREC == MC_PREC_FP64) w.t64 = d.att_thr64[slot];
+        else w.t32 = d.att_thr32[slot];
+    }
+}
+
+// own cell of the colour among the 64
+__device__ __forceinline__ int cache_own(int colour)
+{
+    return 16 * (1 + ((colour >> 2) & 1)) + 4 * (1 + ((colour >> 1) & 1)) + 1 + (colour & 1);
+}
+
+// replica and cell block of active cell g (once per launch, one thread)
+__device__ inline void cache_cell(const DevState &d, int g, CellCache &cc)
+{
+    const int2 sl = d.act_slot ? d.act_slot[g] : make_int2(0, g);
+    cc.r = sl.x;
+    cc.ri = d.rep[sl.x];
+    cc.par = d.par[sl.x];
+    const int h2 = cc.ri.nc >> 1;
+    cc.ax = sl.y % h2;
+    cc.ay = (sl.y / h2) % h2;
+    cc.az = sl.y / (h2 * h2);
+}
+
+// the sweep's grid shift and extents (T threads of the group)
+template <int T>
+__device__ __forceinline__ void cache_sweep(const DevState &d, int gt, CellCache &cc)
+{
+    const int nc = cc.ri.nc;
+    for (int i = gt; i < 64; i += T) {
+        int x = 2 * cc.ax - 1 + (i & 3), y = 2 * cc.ay - 1 + ((i >> 2) & 3), z = 2 * cc.az - 1 + (i >> 4);
+        x += x < 0 ? nc : (x >= nc ? -nc : 0);
+        y += y < 0 ? nc : (y >= nc ? -nc : 0);
+        z += z < 0 ? nc : (z >= nc ? -nc : 0);
+        const int c = cc.ri.cell_off + (z * nc + y) * nc + x;
+        const int a = d.cell_start[c];
+        cc.ext[i] = make_int4(a, d.cell_start[c + 1] - a, c, 0);
+    }
+    if (gt < 3) cc.shift[gt] = d.ctr[cc.r].shift[gt];
+}
+
 // All n attempts of active cell g of the colour, by the 32 W threads of one
 // group (group index gid within the block, its shared memory at gsmem).
-template <int PREC, int W>
+// CACHED: cc holds the group's cells (g is not read).
+template <int PREC, int W, bool CACHED>
 __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &lg, int g, const ModelDev &md,
-                         const MixDev &mx, unsigned char *gsmem, int gid, unsigned dep)
+                         const MixDev &mx, unsigned char *gsmem, int gid, unsigned dep, const CellCache *cc)
 {
     constexpr int T = 32 * W;          // threads per cell
     const int gt = threadIdx.x % T;
@@ -1370,16 +1446,34 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
     const WarpScr S = warp_scr(G, wig);
 
     // ---- which cell ----
-    const int2 sl = d.act_slot ? d.act_slot[g] : make_int2(0, g);
-    const int r = sl.x;
-    const RepInfo ri = d.rep[r];
-    const RepParam dy = d.par[r];
-    const RepCtr ct = d.ctr[r];
-    const int nc = ri.nc, h2 = nc >> 1;
-    const int a_loc = sl.y;
-    const int cx = 2 * (a_loc % h2) + (colour & 1);
-    const int cy = 2 * ((a_loc / h2) % h2) + ((colour >> 1) & 1);
-    const int cz = 2 * (a_loc / (h2 * h2)) + ((colour >> 2) & 1);
+    int r, ax, ay, az;
+    RepInfo ri;
+    RepParam dy;
+    uint32_t shift[3];
+    if constexpr (CACHED) {
+        r = cc->r;
+        ri = cc->ri;
+        dy = cc->par;
+        ax = cc->ax;
+        ay = cc->ay;
+        az = cc->az;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) shift[k] = cc->shift[k];
+    } else {
+        const int2 sl = d.act_slot ? d.act_slot[g] : make_int2(0, g);
+        r = sl.x;
+        ri = d.rep[r];
+        dy = d.par[r];
+        const RepCtr ct = d.ctr[r];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) shift[k] = ct.shift[k];
+        const int h2 = ri.nc >> 1;
+        ax = sl.y % h2;
+        ay = (sl.y / h2) % h2;
+        az = sl.y / (h2 * h2);
+    }
+    const int nc = ri.nc;
+    const int cx = 2 * ax + (colour & 1), cy = 2 * ay + ((colour >> 1) & 1), cz = 2 * az + ((colour >> 2) & 1);
     const int cellL = (cz * nc + cy) * nc + cx;
     const int cellG = ri.cell_off + cellL;
     const bool raw = nc == 2;
@@ -1388,9 +1482,7 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
     // ---- neighbourhood: own cell first.  The extents of the cells and the
     // random words of the first 32 attempts are loaded before waiting for the
     // neighbours (both are fixed for the sweep); the records only after ----
-    uint4 rb0 = make_uint4(0, 0, 0, 0), rb1 = rb0;   // warp 0: attempt `lane`'s draws
-    double th64 = 0.0;
-    float th32 = 0.f;
+    Draws pf{};                        // warp 0: attempt `lane`'s draws
     if (wig == 0) {
         int cnt = 0, cst = 0, wait_c = -1;
         unsigned wait_n = 0;
@@ -1402,9 +1494,18 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
                 const int kk = (lane == 0) ? 13 : (lane <= 13 ? lane - 1 : lane);   // 13 = (0,0,0)
                 ox = kk % 3 - 1; oy = (kk / 3) % 3 - 1; oz = kk / 9 - 1;
             }
-            const int nx = (cx + ox + nc) % nc, ny = (cy + oy + nc) % nc, nz = (cz + oz + nc) % nc;
-            const int c = ri.cell_off + (nz * nc + ny) * nc + nx;
-            const int ncol = (nx & 1) | ((ny & 1) << 1) | ((nz & 1) << 2);
+            int c;
+            if constexpr (CACHED) {
+                const int4 e = cc->ext[cache_own(colour) + 16 * oz + 4 * oy + ox];
+                cst = e.x;
+                cnt = e.y;
+                c = e.z;
+            } else {
+                const int nx = (cx + ox + nc) % nc, ny = (cy + oy + nc) % nc, nz = (cz + oz + nc) % nc;
+                c = ri.cell_off + (nz * nc + ny) * nc + nx;
+            }
+            // (n_c is even: a neighbour's colour is the parity of the sums)
+            const int ncol = ((cx + ox) & 1) | (((cy + oy) & 1) << 1) | (((cz + oz) & 1) << 2);
             if (W == 1) {
                 if (dep != 0 && ncol < colour) wait_c = c;
                 wait_n = dep;
@@ -1412,19 +1513,13 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
                 if (dep != 0) wait_c = c;
                 wait_n = ncol < colour ? 2u * dep : 2u * dep - 1u;
             }
-            cst = d.cell_start[c];
-            cnt = d.cell_start[c + 1] - cst;
-        }
-        {
-            const int n0 = __shfl_sync(FULL, cnt, 0), s0 = __shfl_sync(FULL, cst, 0);
-            if (lane < n0) {
-                const size_t slot = (size_t)s0 + (size_t)lane;
-                rb0 = d.att_rnd[2 * slot];
-                rb1 = d.att_rnd[2 * slot + 1];
-                if (PREC == MC_PREC_FP64) th64 = d.att_thr64[slot];
-                else th32 = d.att_thr32[slot];
+            if constexpr (!CACHED) {
+                cst = d.cell_start[c];
+                cnt = d.cell_start[c + 1] - cst;
             }
         }
+        const int n0 = __shfl_sync(FULL, cnt, 0), s0 = __shfl_sync(FULL, cst, 0);
+        load_draws<PREC>(d, s0, n0, lane, pf);
         // one-warp groups wait before the offsets, multi-warp groups after
         // (each order measured faster for its schedule)
         if (W == 1 && wait_c >= 0) wait_done(d.cell_done + wait_c, wait_n, d.err, d.wait_limit);
@@ -1491,10 +1586,10 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
         if (!ok) G.misc[MS_FAIL] = 1;
         if (lane < n) {
             uint4 *wv = (uint4 *)(G.rnd + 8 * lane);
-            wv[0] = rb0;
-            wv[1] = rb1;
-            if (PREC == MC_PREC_FP64) G.thr64[lane] = th64;
-            else G.thr32[lane] = th32;
+            wv[0] = pf.b0;
+            wv[1] = pf.b1;
+            if (PREC == MC_PREC_FP64) G.thr64[lane] = pf.t64;
+            else G.thr32[lane] = pf.t32;
         }
         if (lane < PADS) G.rec[K + lane] = make_int4(0, 0, 0, PAD_W);
         __syncwarp();
@@ -1534,10 +1629,10 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
         }
         if (wig == 0 && lane < n) {
             uint4 *wv = (uint4 *)(G.rnd + 8 * lane);
-            wv[0] = rb0;
-            wv[1] = rb1;
-            if (PREC == MC_PREC_FP64) G.thr64[lane] = th64;
-            else G.thr32[lane] = th32;
+            wv[0] = pf.b0;
+            wv[1] = pf.b1;
+            if (PREC == MC_PREC_FP64) G.thr64[lane] = pf.t64;
+            else G.thr32[lane] = pf.t32;
         }
         if (gt < PADS) G.rec[K + gt] = make_int4(0, 0, 0, PAD_W);
         gsync<W>(gid);
@@ -1550,9 +1645,9 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
     c.n = n;
     c.cellL = cellL;
     c.nc = nc;
-    c.shift[0] = ct.shift[0];
-    c.shift[1] = ct.shift[1];
-    c.shift[2] = ct.shift[2];
+    c.shift[0] = shift[0];
+    c.shift[1] = shift[1];
+    c.shift[2] = shift[2];
     // origin of the conflict test's frame: any point near the cell will do (the
     // test compares differences with a 1% margin); own atom 0 as staged
     const int4 p0 = n > 0 ? G.rec[0] : make_int4(0, 0, 0, 0);
@@ -1629,7 +1724,7 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
             }
             // committed attempts touch different molecules: each warp applies its own
             if (wig < adv) {
-                if (lane == 0) commit<PREC>(G, R, a + wig, lg, ri, ct.sweep, own_start, d.img);
+                if (lane == 0) commit<PREC>(G, R, a + wig, lg, ri, lg.base ? d.ctr[r].sweep : 0ull, own_start, d.img, d.rec[buf] + own_start);
                 cnt += tally_inc(R, lane);
                 inter_lane += (unsigned)R.inter;
                 if (R.accept) {
@@ -1643,17 +1738,14 @@ __device__ void run_cell(const DevState &d, int buf, int colour, const LogArgs &
         }
     }
 
-    // ---- write back the cell and publish it to the neighbours waiting for
-    // it; then the counts, which nobody waits for: the warps' tallies in warp
+    // ---- publish the cell to the neighbours waiting for it; then the counts, which nobody waits for: the warps' tallies in warp
     // order (one-warp groups reduce their lanes' counts before publishing,
     // multi-warp groups after: each order measured faster for its schedule) ----
-    int4 *dst = d.rec[buf] + own_start;
-    for (int kk = gt; kk < n; kk += T) dst[kk] = G.rec[kk];
     if constexpr (W == 1) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) inter_lane += __shfl_xor_sync(FULL, inter_lane, o);
     }
-    gsync<W>(gid);   // every write-back is done
+    gsync<W>(gid);   // every commit is done
     if (gt == 0 && dep != 0) signal_done(d.cell_done + cellG);
     if constexpr (W > 1) {
 #pragma unroll
@@ -1711,7 +1803,7 @@ __global__ void __launch_bounds__(phase_threads<W>(), W == 1 ? 15 : 1) phase_ker
     __syncthreads();
     const int g = blockIdx.x * CPB + gid;
     if (g >= d.n_act) return;          // whole group leaves together
-    run_cell<PREC, W>(d, buf, colour, lg, g, md, mx, gsmem, gid, 0u);
+    run_cell<PREC, W, false>(d, buf, colour, lg, g, md, mx, gsmem, gid, 0u, nullptr);
 }
 
 // Per replica (one block of at least BLOCK threads): add the sweep's accepted
@@ -1820,7 +1912,8 @@ __device__ __forceinline__ int block_excl_scan(int v, int *tmp, int &total)
     return before + x - v;
 }
 
-template <int PREC, int W>
+// CACHED (W > 1): the grid holds every active cell of a colour, one per group.
+template <int PREC, int W, bool CACHED>
 __global__ void __launch_bounds__(block_threads<W>(), W == 1 ? 3 : 1) sweep_persistent(DevState d, int buf0,
                                                                                      int n_sweeps, GridBar gb)
 {
@@ -1841,6 +1934,10 @@ __global__ void __launch_bounds__(block_threads<W>(), W == 1 ? 3 : 1) sweep_pers
     const int tid = blockIdx.x * NT + threadIdx.x;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const LogArgs none{nullptr, 0, 0};
+    __shared__ CellCache cache[CACHED ? CPB : 1];
+    const int g0 = blockIdx.x * CPB + gid;
+    if (CACHED && g0 < d.n_act && threadIdx.x % T == 0) cache_cell(d, g0, cache[gid]);
+    __syncthreads();
     const int nC = d.n_cells;
     const int chunk = (nC + gridDim.x - 1) / gridDim.x;
     const int lo = min(nC, (int)blockIdx.x * chunk), hi = min(nC, lo + chunk);
@@ -1916,6 +2013,7 @@ __global__ void __launch_bounds__(block_threads<W>(), W == 1 ? 3 : 1) sweep_pers
         } else {
             // (each ordered cell is published in cell_done: no grid-wide
             // barrier before the colours)
+            if (CACHED && g0 < d.n_act) cache_sweep<T>(d, threadIdx.x % T, cache[gid]);
             for (int c = 4 * (blockIdx.x * (NT / 32) + warp); c < nC; c += 4 * gridDim.x * (NT / 32)) {
                 cl_order_cells4(d, buf ^ 1, c, lane);
                 __syncwarp();
@@ -1924,9 +2022,10 @@ __global__ void __launch_bounds__(block_threads<W>(), W == 1 ? 3 : 1) sweep_pers
         }
         // ---- the 8 colours, ordered cell by cell (no grid-wide barrier between
         // colours: each cell waits for its neighbours of smaller colours) ----
+        if (CACHED && g0 < d.n_act) gsync<W>(gid);   // the cache is filled
         for (int colour = 0; colour < 8; ++colour)
-            for (int g = blockIdx.x * CPB + gid; g < d.n_act; g += gridDim.x * CPB)
-                run_cell<PREC, W>(d, buf ^ 1, colour, none, g, md, mx, gsmem, gid, (unsigned)s + 1u);
+            for (int g = g0; g < d.n_act; g += gridDim.x * CPB)
+                run_cell<PREC, W, CACHED>(d, buf ^ 1, colour, none, g, md, mx, gsmem, gid, (unsigned)s + 1u, cache + gid);
         if (!grid_sync(gb, bar_target, d.err, d.wait_limit)) return;
         // ---- finalise the sweep and, in the same stage, count the next
         // sweep's cell list (it reads only the positions written back above,
@@ -1977,14 +2076,20 @@ int phase_set_smem_limit(int bytes_needed)
     ok &= set_kernel_smem(phase_kernel<MC_PREC_FP32, 2>, bytes);
     ok &= set_kernel_smem(phase_kernel<MC_PREC_FP32, 4>, bytes);
     ok &= set_kernel_smem(phase_kernel<MC_PREC_FP32, 8>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 1>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 2>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 4>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 8>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 1>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 2>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 4>, bytes);
-    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 8>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 1, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 2, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 2, true>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 4, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 4, true>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 8, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP64, 8, true>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 1, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 2, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 2, true>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 4, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 4, true>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 8, false>, bytes);
+    ok &= set_kernel_smem(sweep_persistent<MC_PREC_FP32, 8, true>, bytes);
     const int full = cudaSharedmemCarveoutMaxShared;
     cudaFuncSetAttribute(finalize_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, full);
     cudaFuncSetAttribute(cl_count_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, full);
@@ -2027,42 +2132,56 @@ void launch_phases(const DevState &d, int buf, int warps_per_cell, const LogArgs
     launch_finalize(d, st);
 }
 
-template <int PREC, int W>
-static void *persistent_fn()
+template <int PREC>
+static void *persistent_fn(int W, bool cached)
 {
-    return (void *)sweep_persistent<PREC, W>;
+    if (W == 1) return (void *)sweep_persistent<PREC, 1, false>;
+    if (cached)
+        return W == 8 ? (void *)sweep_persistent<PREC, 8, true>
+               : W == 4 ? (void *)sweep_persistent<PREC, 4, true>
+                        : (void *)sweep_persistent<PREC, 2, true>;
+    return W == 8 ? (void *)sweep_persistent<PREC, 8, false>
+           : W == 4 ? (void *)sweep_persistent<PREC, 4, false>
+                    : (void *)sweep_persistent<PREC, 2, false>;
 }
 
-static void *persistent_kernel(int prec, int W)
+static void *persistent_kernel(int prec, int W, bool cached)
 {
-    if (prec == MC_PREC_FP64)
-        return W == 8 ? persistent_fn<MC_PREC_FP64, 8>()
-               : W == 4 ? persistent_fn<MC_PREC_FP64, 4>()
-               : W == 2 ? persistent_fn<MC_PREC_FP64, 2>()
-                        : persistent_fn<MC_PREC_FP64, 1>();
-    return W == 8 ? persistent_fn<MC_PREC_FP32, 8>()
-           : W == 4 ? persistent_fn<MC_PREC_FP32, 4>()
-           : W == 2 ? persistent_fn<MC_PREC_FP32, 2>()
-                    : persistent_fn<MC_PREC_FP32, 1>();
+    return prec == MC_PREC_FP64 ? persistent_fn<MC_PREC_FP64>(W, cached) : persistent_fn<MC_PREC_FP32>(W, cached);
 }
+
+// cells per block of the persistent kernel
+static int persistent_cells(int W) { return (W > 4 ? 32 * W : BLOCK) / (32 * W); }
+
+// whether a grid's groups have one active cell of a colour each
+static bool persistent_cached(const DevState &d, int W, int grid) { return W > 1 && d.n_act <= grid * persistent_cells(W); }
 
 int persistent_grid(const DevState &d, int warps_per_cell, int max_blocks)
 {
-    int dev = 0, sms = 0, coop = 0, per_sm = 0;
+    int dev = 0, sms = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     if (!coop) return 0;
     const size_t sm = phase_smem_bytes(d.stencil_cap, warps_per_cell);
     const int nt = warps_per_cell > 4 ? 32 * warps_per_cell : BLOCK;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel(d.precision, warps_per_cell), nt, sm) !=
-        cudaSuccess)
-        return 0;
     // one block per group of active cells: blocks without a cell would only
     // add arrivals to every grid barrier
-    const int cpb = nt / (32 * warps_per_cell);
+    const int cpb = persistent_cells(warps_per_cell);
     const int needed = std::max((d.n_act + cpb - 1) / cpb, 32);
-    return std::max(0, std::min(std::min(per_sm * sms, needed), max_blocks));
+    auto fits = [&](bool cached) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_kernel(d.precision, warps_per_cell, cached),
+                                                          nt, sm) != cudaSuccess)
+            return 0;
+        return std::max(0, std::min(std::min(per_sm * sms, needed), max_blocks));
+    };
+    // (a grid of either kernel that holds every cell is one of the other's size:
+    // launch_persistent takes the cached kernel for it, so it has to fit there)
+    const int with = warps_per_cell > 1 ? fits(true) : 0;
+    if (with > 0 && persistent_cached(d, warps_per_cell, with)) return with;
+    const int without = fits(false);
+    return persistent_cached(d, warps_per_cell, without) ? with : without;
 }
 
 int launch_persistent(const DevState &d, int buf, int n_sweeps, int warps_per_cell, int grid, unsigned int *bar,
@@ -2073,8 +2192,9 @@ int launch_persistent(const DevState &d, int buf, int n_sweeps, int warps_per_ce
     DevState dd = d;
     void *args[] = {(void *)&dd, (void *)&buf, (void *)&n_sweeps, (void *)&gb};
     const int nt = warps_per_cell > 4 ? 32 * warps_per_cell : BLOCK;
-    const cudaError_t e = cudaLaunchCooperativeKernel(persistent_kernel(d.precision, warps_per_cell), dim3(grid),
-                                                      dim3(nt), args, sm, st);
+    const cudaError_t e = cudaLaunchCooperativeKernel(
+        persistent_kernel(d.precision, warps_per_cell, persistent_cached(d, warps_per_cell, grid)), dim3(grid), dim3(nt),
+        args, sm, st);
     return e == cudaSuccess ? 0 : (int)e;
 }
 
