@@ -673,19 +673,15 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
     // staging capacity: the neighbourhood (mean + 6 sigma + 32) plus the padding records, a multiple of 32
     int cap = o.stencil_cap > 0 ? o.stencil_cap : ((int)std::ceil(max_stencil) + kPadSlots + 31) / 32 * 32;
     h->stencil_cap = cap;
-    // warps per cell: as many as leave every active cell of a colour resident at
-    // once (two blocks of 128 threads per SM at the multi-warp kernels' registers:
-    // 304 cells with four warps, 608 with two); a second round of cells costs more
-    // than the warps save.  us a sweep with 1 / 2 / 4 warps: 216 cells 91 / 69 / 65,
-    // 343 cells 90 / 69 / 99, 512 cells 96 / 76 / 112, 729 cells 98 / 117 / 145,
-    // 1331 cells 114 / 180 / 243; FP64 chains alike
+    // warps per cell: spread small grids over more warps so that every SM has
+    // work; large grids keep one warp per cell (enough cells to fill the GPU)
     if (o.warps_per_cell != 0 && o.warps_per_cell != 1 && o.warps_per_cell != 2 && o.warps_per_cell != 4 &&
         o.warps_per_cell != 8) {
         delete h;
         return fail(MC_ERR_INVALID_ARG, "warps_per_cell must be 0, 1, 2, 4 or 8");
     }
     if (o.warps_per_cell > 0) h->wpb = o.warps_per_cell;
-    else h->wpb = h->n_act > 152 * 4 ? 1 : (h->n_act > 152 * 2 ? 2 : 4);
+    else h->wpb = h->n_act >= 152 * 12 ? 1 : (h->n_act >= 152 * 3 ? 2 : 4);
     h->smem_bytes = phase_smem_bytes(cap, h->wpb);
     if (h->smem_bytes > 220u * 1024u) {
         delete h;
