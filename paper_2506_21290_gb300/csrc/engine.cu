@@ -115,28 +115,34 @@ struct mc_handle {
     double *d_drift = nullptr;           // per replica: last and largest relative drift
     mc_params params{};
     std::vector<RepInfo> reps;
-    // page-locked host staging of the state's uploads and downloads, grown on
-    // demand (pageable memory when page-locked memory cannot be had)
-    void *pin = nullptr;
-    size_t pin_bytes = 0;
-    std::vector<unsigned char> pageable;
-    void *host_buf(size_t bytes)
-    {
-        if (pin && pin_bytes >= bytes) return pin;
-        if (pin) {
-            cudaFreeHost(pin);
+    // page-locked host memory, grown on demand and kept with the handle (pageable
+    // when page-locked memory cannot be had): the staging of the state's uploads
+    // and downloads, and the place where calls receive their results
+    struct HostMem {
+        void *pin = nullptr;
+        size_t bytes = 0;
+        std::vector<unsigned char> pageable;
+        void *get(size_t n)
+        {
+            if (pin && bytes >= n) return pin;
+            release();
+            if (cudaHostAlloc(&pin, n, cudaHostAllocDefault) == cudaSuccess) {
+                bytes = n;
+                return pin;
+            }
             pin = nullptr;
-            pin_bytes = 0;
+            cudaGetLastError();
+            pageable.resize(n);
+            return pageable.data();
         }
-        if (cudaHostAlloc(&pin, bytes, cudaHostAllocDefault) == cudaSuccess) {
-            pin_bytes = bytes;
-            return pin;
+        void release()
+        {
+            if (pin) cudaFreeHost(pin);
+            pin = nullptr;
+            bytes = 0;
         }
-        pin = nullptr;
-        cudaGetLastError();
-        pageable.resize(bytes);
-        return pageable.data();
-    }
+    } staging, results;
+    void *host_buf(size_t bytes) { return staging.get(bytes); }
     // device workspace of the analysis calls, grown on demand and kept with the
     // handle; a call lays its arrays out in it anew
     void *work = nullptr;
@@ -460,16 +466,48 @@ int pack_records(mc_handle *h, const double *xyz, const uint32_t *qfix, const in
     return fail(MC_ERR_BAD_STATE, "non-finite position");
 }
 
-int check_device_errors(mc_handle *h)
-{
-    int e = 0;
-    CUDA_TRY(cudaMemcpyAsync(&e, h->ds.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    if (e & ERR_STENCIL) return fail(MC_ERR_CELL_OVERFLOW, "a cell neighbourhood exceeded the staging capacity");
-    if (e & ERR_TERMS) return fail(MC_ERR_CELL_OVERFLOW, "too many nonzero FP64 terms in one move");
-    if (e & ERR_TIMEOUT) return fail(MC_ERR_TIMEOUT, "a device wait timed out");
-    return MC_OK;
-}
+// The results of one call, in page-locked memory: copies enqueued on the
+// stream, then finish(), which also fetches the device's error word and waits, once
+// (a copy to pageable memory and a wait for each result cost 5 to 10 us apiece).
+class Results {
+public:
+    Results(mc_handle *h, size_t bytes) : h_(h), base_((unsigned char *)h->results.get(bytes + 256)) {}
+    // n values from device memory; valid after finish()
+    template <class T>
+    const T *get(const T *dev, size_t n)
+    {
+        T *to = (T *)(base_ + used_);
+        used_ += (n * sizeof(T) + 15) & ~(size_t)15;
+        const cudaError_t e = cudaMemcpyAsync(to, dev, n * sizeof(T), cudaMemcpyDeviceToHost, h_->stream);
+        if (failed_ == cudaSuccess) failed_ = e;
+        return to;
+    }
+    int wait()
+    {
+        CUDA_TRY(failed_);
+        CUDA_TRY(cudaStreamSynchronize(h_->stream));
+        return MC_OK;
+    }
+    int finish()
+    {
+        const int *err = get(h_->ds.err, 1);
+        const int rc = wait();
+        if (rc) return rc;
+        const int e = *err;
+        if (e & ERR_STENCIL) return fail(MC_ERR_CELL_OVERFLOW, "a cell neighbourhood exceeded the staging capacity");
+        if (e & ERR_TERMS) return fail(MC_ERR_CELL_OVERFLOW, "too many nonzero FP64 terms in one move");
+        if (e & ERR_TIMEOUT) return fail(MC_ERR_TIMEOUT, "a device wait timed out");
+        return MC_OK;
+    }
+
+private:
+    mc_handle *h_;
+    unsigned char *base_;
+    size_t used_ = 0;
+    cudaError_t failed_ = cudaSuccess;
+};
+
+int check_device_errors(mc_handle *h) { return Results(h, 0).finish(); }
 
 // energy of each replica into h->d_e_out (device)
 int enqueue_energy(mc_handle *h)
@@ -494,11 +532,9 @@ int rebuild_and_reset(mc_handle *h, const int4 *rec, const std::vector<int> *img
     int rc = enqueue_energy(h);
     if (rc) return rc;
     CUDA_TRY(cudaMemcpyAsync(h->ds.e_run, h->d_e_out, sizeof(double) * h->n_rep, cudaMemcpyDeviceToDevice, h->stream));
-    std::vector<double> e(h->n_rep);
-    CUDA_TRY(cudaMemcpyAsync(e.data(), h->d_e_out, sizeof(double) * h->n_rep, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    rc = check_device_errors(h);
-    if (rc) return rc;
+    Results res(h, sizeof(double) * h->n_rep);
+    const double *e = res.get(h->d_e_out, h->n_rep);
+    if ((rc = res.finish())) return rc;
     for (int r = 0; r < h->n_rep; ++r)
         if (!std::isfinite(e[r])) return fail(MC_ERR_BAD_STATE, "non-finite energy in replica " + std::to_string(r));
     h->has_t0 = false;
@@ -803,7 +839,10 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         return fail(MC_ERR_INVALID_ARG, "persistent sweeps need cooperative launch support");
     }
     int4 *rec = (int4 *)h->host_buf(sizeof(int4) * (size_t)h->n_sites);
-    rc = pack_records(h, xyz, nullptr, types, rec);
+    // room for the per-particle results and wavevector tables of the analysis calls
+    h->results.get(((size_t)64 << 10) + sizeof(double) * ((size_t)h->n_sites + 2 * (size_t)M_tot + 3 * (size_t)n_rep));
+    rc = h->need_work(std::min<size_t>((size_t)8 << 20, ((size_t)64 << 10) + 512 * sizeof(Turns) * (size_t)n_rep));
+    if (rc == MC_OK) rc = pack_records(h, xyz, nullptr, types, rec);
     if (rc == MC_OK) rc = rebuild_and_reset(h, rec);
     if (rc) {
         std::string msg = g_err;
@@ -861,7 +900,8 @@ void mc_destroy(mc_handle *h)
         if (h->graph[b]) cudaGraphExecDestroy(h->graph[b]);
     for (auto &a : h->allocs) cudaFree(a.p);
     if (h->work) cudaFree(h->work);
-    if (h->pin) cudaFreeHost(h->pin);
+    h->staging.release();
+    h->results.release();
     if (h->own_stream) cudaStreamDestroy(h->own_stream);
     delete h;
 }
@@ -1102,9 +1142,10 @@ int mc_sync(mc_handle *h)
     if (!h) return fail(MC_ERR_INVALID_ARG, "NULL handle");
     int rc = set_device(h);
     if (rc) return rc;
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    rc = check_device_errors(h);
+    if (rc) return rc;
     CUDA_TRY(cudaGetLastError());
-    return check_device_errors(h);
+    return MC_OK;
 }
 
 int mc_energy(mc_handle *h, double *E_out)
@@ -1113,9 +1154,11 @@ int mc_energy(mc_handle *h, double *E_out)
     int rc = set_device(h);
     if (rc) return rc;
     if ((rc = enqueue_energy(h))) return rc;
-    CUDA_TRY(cudaMemcpyAsync(E_out, h->d_e_out, sizeof(double) * h->n_rep, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    return check_device_errors(h);
+    Results res(h, sizeof(double) * h->n_rep);
+    const double *e = res.get(h->d_e_out, h->n_rep);
+    rc = res.finish();
+    std::memcpy(E_out, e, sizeof(double) * h->n_rep);
+    return rc;
 }
 
 int mc_pressure(mc_handle *h, const double *T, double *out)
@@ -1127,15 +1170,15 @@ int mc_pressure(mc_handle *h, const double *T, double *out)
     if (rc) return rc;
     launch_virial(h->ds, h->cur, h->d_e_site, h->d_e_out, h->stream);
     CUDA_TRY(cudaGetLastError());
-    std::vector<double> w(h->n_rep);
-    CUDA_TRY(cudaMemcpyAsync(w.data(), h->d_e_out, sizeof(double) * h->n_rep, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    Results res(h, sizeof(double) * h->n_rep);
+    const double *w = res.get(h->d_e_out, h->n_rep);
+    rc = res.finish();
     for (int r = 0; r < h->n_rep; ++r) {
         const double V = h->reps[r].L * h->reps[r].L * h->reps[r].L;
         out[2 * r] = w[r];
         out[2 * r + 1] = (double)h->reps[r].n_sites * T[r] / V + w[r] / (3.0 * V);
     }
-    return check_device_errors(h);
+    return rc;
 }
 
 int mc_cell_grid(double L, int n_mol, const int32_t *types, const mc_params *params, int request, int *nc_out,
@@ -1179,9 +1222,11 @@ int mc_structure_factor(mc_handle *h, const double *qvec, int n_q, double *out)
         launch_sq(h->ds, h->cur, turns, n, max_sites, part, dout + k, n_q, h->stream);
     }
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(out, dout, b_out, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    return check_device_errors(h);
+    Results res(h, b_out);
+    const double *got = res.get(dout, (size_t)n_q * R);
+    rc = res.finish();
+    std::memcpy(out, got, b_out);
+    return rc;
 }
 
 int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, double *g)
@@ -1202,8 +1247,10 @@ int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, dou
     CUDA_TRY(cudaMemsetAsync(dc, 0, sizeof(unsigned long long) * n, h->stream));
     launch_pair_hist(h->ds, h->cur, max_sites, dr, n_bins, dc, h->stream);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(counts, dc, sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    Results res(h, sizeof(unsigned long long) * n);
+    const unsigned long long *got = res.get(dc, n);
+    rc = res.finish();
+    std::memcpy(counts, got, sizeof(unsigned long long) * n);
     if (g) {
         // g(r) at the bin centres: 2 counts / (N rho shell volume), rho = N / V
         const double pi = 3.14159265358979323846;
@@ -1216,11 +1263,11 @@ int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, dou
             }
         }
     }
-    return check_device_errors(h);
+    return rc;
 }
 
 // the records (cell order) and, when img is asked for, the image counts (site
-// order), into the handle's host staging
+// order), on their way into the handle's host staging (there after a finish())
 static int fetch_records(mc_handle *h, const int4 **rec, const int **img)
 {
     const size_t n = (size_t)h->n_sites;
@@ -1229,10 +1276,9 @@ static int fetch_records(mc_handle *h, const int4 **rec, const int **img)
     if (img)
         CUDA_TRY(cudaMemcpyAsync(buf + sizeof(int4) * n, h->ds.img, sizeof(int) * 3 * n, cudaMemcpyDeviceToHost,
                                  h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
     *rec = (const int4 *)buf;
     if (img) *img = (const int *)(buf + sizeof(int4) * n);
-    return check_device_errors(h);
+    return MC_OK;
 }
 
 static int site_of(const mc_handle *h, int r, const int4 &v)
@@ -1245,9 +1291,20 @@ int mc_state(mc_handle *h, double *xyz_out, int32_t *types_out, mc_stats *stats_
     if (!h) return fail(MC_ERR_INVALID_ARG, "NULL handle");
     int rc = set_device(h);
     if (rc) return rc;
-    if (xyz_out || types_out) {
-        const int4 *rec = nullptr;
-        if ((rc = fetch_records(h, &rec, nullptr))) return rc;
+    const size_t R = (size_t)h->n_rep;
+    const int4 *rec = nullptr;
+    if ((xyz_out || types_out) && (rc = fetch_records(h, &rec, nullptr))) return rc;
+    Results res(h, R * (STAT_N * sizeof(unsigned long long) + 3 * sizeof(double)) + 64);
+    const unsigned long long *st = nullptr;
+    const double *e = nullptr, *dr = nullptr;
+    if (stats_out) {
+        st = res.get(h->ds.stats, STAT_N * R);
+        e = res.get(h->ds.e_run, R);
+        dr = res.get(h->d_drift, 2 * R);
+    }
+    if (!rec && !stats_out) return MC_OK;
+    if ((rc = res.finish()) && rec) return rc;
+    if (rec) {
         // on host threads, each taking a run of record slots (a replica's
         // records fill the slots of its sites; each record writes its own site)
         host_parallel((size_t)h->n_sites, 65536, [&](size_t b, size_t e) {
@@ -1269,16 +1326,9 @@ int mc_state(mc_handle *h, double *xyz_out, int32_t *types_out, mc_stats *stats_
         });
     }
     if (stats_out) {
-        std::vector<unsigned long long> st((size_t)STAT_N * h->n_rep);
-        std::vector<double> e(h->n_rep), dr(2 * (size_t)h->n_rep);
-        CUDA_TRY(cudaMemcpyAsync(st.data(), h->ds.stats, sizeof(unsigned long long) * st.size(), cudaMemcpyDeviceToHost,
-                                 h->stream));
-        CUDA_TRY(cudaMemcpyAsync(e.data(), h->ds.e_run, sizeof(double) * h->n_rep, cudaMemcpyDeviceToHost, h->stream));
-        CUDA_TRY(cudaMemcpyAsync(dr.data(), h->d_drift, sizeof(double) * dr.size(), cudaMemcpyDeviceToHost, h->stream));
-        CUDA_TRY(cudaStreamSynchronize(h->stream));
         for (int r = 0; r < h->n_rep; ++r) {
             mc_stats &s = stats_out[r];
-            const unsigned long long *v = st.data() + (size_t)STAT_N * r;
+            const unsigned long long *v = st + (size_t)STAT_N * r;
             for (int k = 0; k < 4; ++k) {
                 s.attempts[k] = v[STAT_ATT + k];
                 s.accepts[k] = v[STAT_ACC + k];
@@ -1294,9 +1344,8 @@ int mc_state(mc_handle *h, double *xyz_out, int32_t *types_out, mc_stats *stats_
             s.drift_last = dr[2 * (size_t)r];
             s.drift_max = dr[2 * (size_t)r + 1];
         }
-        return check_device_errors(h);
     }
-    return MC_OK;
+    return rc;
 }
 
 int mc_state_fixed(mc_handle *h, uint32_t *q_out, int64_t *X_out, int32_t *types_out)
@@ -1306,7 +1355,7 @@ int mc_state_fixed(mc_handle *h, uint32_t *q_out, int64_t *X_out, int32_t *types
     if (rc) return rc;
     const int4 *rec = nullptr;
     const int *img = nullptr;
-    if ((rc = fetch_records(h, &rec, &img))) return rc;
+    if ((rc = fetch_records(h, &rec, &img)) || (rc = check_device_errors(h))) return rc;
     for (int r = 0; r < h->n_rep; ++r) {
         const RepInfo &ri = h->reps[r];
         for (int i = 0; i < ri.n_sites; ++i) {
@@ -1401,21 +1450,27 @@ int mc_observables(mc_handle *h, const double *qvec_atom, int n_qa, const double
     if ((rc = h->need_work(b_t + sizeof(double) * 3 * (n_qa + n_qc)))) return rc;
     Turns *ta = (Turns *)h->work, *tc = ta + R * n_qa;
     double *dqa = (double *)(tc + R * n_qc), *dqc = dqa + 3 * n_qa;
-    CUDA_TRY(cudaMemcpyAsync(dqa, qvec_atom, sizeof(double) * 3 * n_qa, cudaMemcpyHostToDevice, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(dqc, qvec_cm, sizeof(double) * 3 * n_qc, cudaMemcpyHostToDevice, h->stream));
+    const size_t b_qa = sizeof(double) * 3 * n_qa, b_qc = sizeof(double) * 3 * n_qc;
+    unsigned char *hq = (unsigned char *)h->host_buf(b_qa + b_qc);
+    std::memcpy(hq, qvec_atom, b_qa);
+    std::memcpy(hq + b_qa, qvec_cm, b_qc);
+    CUDA_TRY(cudaMemcpyAsync(dqa, hq, b_qa + b_qc, cudaMemcpyHostToDevice, h->stream));
     launch_turns(h->ds, dqa, n_qa, false, ta, h->stream);
     launch_turns(h->ds, dqc, n_qc, true, tc, h->stream);
     launch_gather(h->ds, h->cur, h->d_X, h->d_types, h->stream);
     launch_observables(h->ds, h->d_X, h->obs, h->chunks, ta, n_qa, tc, n_qc, h->d_fs, h->d_fscm, h->d_c2,
                        h->d_obs_part, h->d_obs_out, h->stream);
     CUDA_TRY(cudaGetLastError());
-    CUDA_TRY(cudaMemcpyAsync(out, h->d_obs_out, sizeof(double) * 3 * h->n_rep, cudaMemcpyDeviceToHost, h->stream));
-    const size_t M = (size_t)h->n_sites / 3;
-    if (fs_atom)
-        CUDA_TRY(cudaMemcpyAsync(fs_atom, h->d_fs, sizeof(double) * h->n_sites, cudaMemcpyDeviceToHost, h->stream));
-    if (fscm_mol) CUDA_TRY(cudaMemcpyAsync(fscm_mol, h->d_fscm, sizeof(double) * M, cudaMemcpyDeviceToHost, h->stream));
-    if (c2_mol) CUDA_TRY(cudaMemcpyAsync(c2_mol, h->d_c2, sizeof(double) * M, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    const size_t N = (size_t)h->n_sites, M = N / 3;
+    Results res(h, sizeof(double) * (3 * R + N + 2 * M));
+    const double *mean = res.get(h->d_obs_out, 3 * R);
+    const double *fs = fs_atom ? res.get(h->d_fs, N) : nullptr, *fcm = fscm_mol ? res.get(h->d_fscm, M) : nullptr,
+                 *c2 = c2_mol ? res.get(h->d_c2, M) : nullptr;
+    if ((rc = res.wait())) return rc;
+    std::memcpy(out, mean, sizeof(double) * 3 * R);
+    if (fs) std::memcpy(fs_atom, fs, sizeof(double) * N);
+    if (fcm) std::memcpy(fscm_mol, fcm, sizeof(double) * M);
+    if (c2) std::memcpy(c2_mol, c2, sizeof(double) * M);
     return MC_OK;
 }
 
@@ -1909,14 +1964,13 @@ int mc_md_state(mc_handle *h, double *v_out, double *out)
     int rc = set_device(h);
     if (rc) return rc;
     const int R = h->n_rep;
-    std::vector<double> v(3 * (size_t)h->n_sites), xi(R), eta(R), U(R);
+    const size_t nv = 3 * (size_t)h->n_sites;
     if ((rc = enqueue_energy(h))) return rc;
-    CUDA_TRY(cudaMemcpyAsync(v.data(), h->md.dev.v, sizeof(double) * v.size(), cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(xi.data(), h->md.dev.xi, sizeof(double) * R, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(eta.data(), h->md.dev.eta, sizeof(double) * R, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaMemcpyAsync(U.data(), h->d_e_out, sizeof(double) * R, cudaMemcpyDeviceToHost, h->stream));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    if (v_out) std::memcpy(v_out, v.data(), sizeof(double) * v.size());
+    Results res(h, sizeof(double) * (nv + 3 * (size_t)R));
+    const double *v = res.get(h->md.dev.v, nv), *xi = res.get(h->md.dev.xi, R), *eta = res.get(h->md.dev.eta, R),
+                 *U = res.get(h->d_e_out, R);
+    rc = res.finish();
+    if (v_out) std::memcpy(v_out, v, sizeof(double) * nv);
     for (int r = 0; r < R; ++r) {
         double K = 0.0;
         const size_t o = 3 * (size_t)h->reps[r].site_off, n = 3 * (size_t)h->reps[r].n_sites;
@@ -1930,7 +1984,7 @@ int mc_md_state(mc_handle *h, double *v_out, double *out)
         out[5 * r + 3] = eta[r];
         out[5 * r + 4] = K + U[r] + thermo;
     }
-    return check_device_errors(h);
+    return rc;
 }
 
 int mc_get_info(mc_handle *h, mc_info *info)
