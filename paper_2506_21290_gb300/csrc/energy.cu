@@ -42,8 +42,11 @@ __device__ __forceinline__ double walk_ln(double y)
 // pair from its atom of the smaller site index (pair_walk.cuh), FP64.  A warp
 // walks one to four cells and keeps what does not fill a batch of 32 pairs for
 // the next; bonds, whose Eq. 2 costs three times Eq. 1, wait in a ring of their
-// own for full batches.  The sums (per lane, then lanes, warps and blocks) run in
-// a fixed order: the same on every run for a given state.
+// own for full batches.  The sums (per lane, then lanes, warps and, in a second
+// kernel, blocks) run in a fixed order: the same on every run for a given state.
+// (No counter tells a last block to add the blocks' sums: mc_energy_device is
+// asynchronous, so two of these may overlap on two streams, or in two replayed
+// graphs, with one handle's workspace.  Both write the same numbers to it.)
 // Energy of 24000 atoms 41 us (62 with the sum over cells, when every lane of a
 // warp walked a neighbour cell and bonds shared the batches), of 192000 atoms
 // 133 (290), of 256 replicas with 823000 atoms 505 (1161).
@@ -97,21 +100,20 @@ struct EnergyWalk {
 };
 
 template <bool VIRIAL>
-__global__ void __launch_bounds__(32 * kEnergyWarps) pair_energy_kernel(DevState d, int buf, double *part, double *out)
+__global__ void __launch_bounds__(32 * kEnergyWarps) pair_energy_kernel(DevState d, int buf, double *part)
 {
     __shared__ WalkSmem walk[kEnergyWarps];
-    __shared__ double bond_r2[kEnergyWarps][64], red[32 * kEnergyWarps];
+    __shared__ double bond_r2[kEnergyWarps][64], red[kEnergyWarps];
     __shared__ int bond_ab[kEnergyWarps][64];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int r = 0, c0 = 0, b0 = 0;
+    int r = 0, c0 = 0;
     if (d.cells.unit != nullptr) {
         const int2 u = d.cells.unit[blockIdx.x];
         r = u.x;
         c0 = u.y;
-        b0 = d.cells.rep0[r];
     }
     const RepInfo ri = d.rep[r];
-    const int n_cells = ri.nc * ri.nc * ri.nc, per = walk_cells(ri.n_sites, n_cells);
+    const int per = walk_cells(ri.n_sites, ri.nc * ri.nc * ri.nc);
     if (d.cells.unit == nullptr) c0 = blockIdx.x * kEnergyWarps * per;
     const ModelDev &md = *d.model;
     EnergyWalk<VIRIAL> p{md, quantum2(ri.h), 6.0 * md.e4, walk[w].ring, bond_r2[w], bond_ab[w], lane};
@@ -129,15 +131,54 @@ __global__ void __launch_bounds__(32 * kEnergyWarps) pair_energy_kernel(DevState
         for (int k = 1; k < kEnergyWarps; ++k) v = __dadd_rn(v, red[k]);
         part[blockIdx.x] = v;
     }
-    const int nb = n_cells / (kEnergyWarps * per);
-    if (!last_block(d.arrived + r, nb)) return;
-    v = sum_parts<32 * kEnergyWarps>(part + b0, nb, red);
-    if (threadIdx.x == 0) out[r] = v;
+}
+
+// Sum of each replica's parts (one block each), in a fixed order: thread t adds
+// parts t, t + 256, ..., eight loads in flight; then a tree.
+constexpr int kPartsThreads = 256;
+
+__global__ void __launch_bounds__(kPartsThreads) replica_parts_kernel(DevState d, const double *part, double *out)
+{
+    const int r = blockIdx.x, tid = threadIdx.x;
+    const int b0 = d.cells.unit != nullptr ? d.cells.rep0[r] : 0;
+    const int nb = d.cells.unit != nullptr ? d.cells.rep0[r + 1] - b0 : d.cells.n;
+    const double *p = part + b0;
+    double s = 0.0;
+    for (int k = tid; k < nb; k += 8 * kPartsThreads) {
+        double v[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = k + j * kPartsThreads < nb ? p[k + j * kPartsThreads] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (k + j * kPartsThreads < nb) s = __dadd_rn(s, v[j]);
+    }
+    __shared__ double red[kPartsThreads];
+    red[tid] = s;
+    __syncthreads();
+    if (tid < 64) red[tid] = __dadd_rn(__dadd_rn(red[tid], red[tid + 64]), __dadd_rn(red[tid + 128], red[tid + 192]));
+    __syncthreads();
+    for (int o = 32; o > 0; o >>= 1) {
+        if (tid < o) red[tid] = __dadd_rn(red[tid], red[tid + o]);
+        __syncthreads();
+    }
+    if (tid == 0) out[r] = red[0];
+}
+
+template <bool VIRIAL>
+static void launch_walk(const DevState &d, int buf, double *part, double *out, cudaStream_t st)
+{
+    pair_energy_kernel<VIRIAL><<<d.cells.n, 32 * kEnergyWarps, 0, st>>>(d, buf, part);
+    replica_parts_kernel<<<d.n_rep, kPartsThreads, 0, st>>>(d, part, out);
 }
 
 void launch_energy(const DevState &d, int buf, double *part, double *e_out_dev, cudaStream_t st)
 {
-    pair_energy_kernel<false><<<d.cells.n, 32 * kEnergyWarps, 0, st>>>(d, buf, part, e_out_dev);
+    launch_walk<false>(d, buf, part, e_out_dev, st);
+}
+
+void launch_virial(const DevState &d, int buf, double *part, double *w_out_dev, cudaStream_t st)
+{
+    launch_walk<true>(d, buf, part, w_out_dev, st);
 }
 
 // Drift check of the running total against a fresh FP64 recompute E, per
@@ -159,11 +200,6 @@ __global__ void drift_kernel(DevState d, const double *E, double *drift)
 void launch_drift(const DevState &d, const double *E, double *drift, cudaStream_t st)
 {
     drift_kernel<<<(d.n_rep + 127) / 128, 128, 0, st>>>(d, E, drift);
-}
-
-void launch_virial(const DevState &d, int buf, double *part, double *w_out_dev, cudaStream_t st)
-{
-    pair_energy_kernel<true><<<d.cells.n, 32 * kEnergyWarps, 0, st>>>(d, buf, part, w_out_dev);
 }
 
 // Unwrapped fixed-point positions and types in site-index order.

@@ -778,7 +778,6 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         (rc = h->alloc(&h->d_c2, M_tot)) || (rc = h->alloc(&d_m0, chunk_m0.size())) ||
         (rc = h->alloc(&d_c0, rep_chunk0.size())) ||
         (rc = h->alloc(&d_cells, cell_units.unit.size())) || (rc = h->alloc(&d_cells0, cell_units.rep0.size())) ||
-        (rc = h->alloc(&d.arrived, n_rep)) ||
         (rc = h->alloc(&h->d_obs_part, (chunk_m0.size() - 1) * kCorrPart)) ||
         (rc = h->alloc(&h->d_obs_out, 3 * (size_t)n_rep)) ||
         (rc = h->alloc(&h->ds.att_rnd, 2 * (size_t)h->n_sites)) || (rc = h->alloc(&h->d_bar, 2)) ||
@@ -1887,10 +1886,10 @@ int mc_md_setup(mc_handle *h, double dt, double tau_T, const double *T, const do
     });
     const size_t nu = units.unit.size();
     double *bufs[10] = {};
-    const size_t sizes[12] = {3 * N, 3 * N, R, R, R, R, R, R, R, nu, nu, R + 1};
+    const size_t sizes[13] = {3 * N, 3 * N, R, R, R, R, R, R, R, nu, nu, R + 1, R};
     int2 *d_unit = nullptr;
     int *d_unit0 = nullptr;
-    for (int k = 0; k < 12; ++k) {
+    for (int k = 0; k < 13; ++k) {
         void *p = nullptr;
         const size_t bytes = sizes[k] * (k < 10 ? sizeof(double) : k == 10 ? sizeof(int2) : sizeof(int));
         cudaError_t e = cudaMalloc(&p, bytes);
@@ -1902,7 +1901,8 @@ int mc_md_setup(mc_handle *h, double dt, double tau_T, const double *T, const do
         CUDA_TRY(cudaMemsetAsync(p, 0, bytes, h->stream));
         if (k < 10) bufs[k] = (double *)p;
         else if (k == 10) d_unit = (int2 *)p;
-        else d_unit0 = (int *)p;
+        else if (k == 11) d_unit0 = (int *)p;
+        else m.dev.arrived = (unsigned *)p;
     }
     m.dev.v = bufs[0];
     m.dev.F = bufs[1];

@@ -114,7 +114,6 @@ struct DevState {
     const MixDev *mix;
     const int *rep_of_site;
     Units cells;         // blocks of kEnergyWarps x walk_cells cells (energy walks; pair_walk.cuh)
-    unsigned *arrived;   // per replica: blocks of a walk that have written their sum (zero between launches)
     const int *act_off;  // n_rep + 1 prefix of (nc/2)^3
     const int2 *act_slot;    // per active-cell slot of a colour (n_act), in schedule order: {replica, active
                              // cell within the replica}; null for one replica (slot = active cell)

@@ -99,6 +99,45 @@ __device__ __forceinline__ double md_second_kick(const MdDev &m, size_t o, doubl
     return __dmul_rn(v, v);
 }
 
+// Fixed-order sum over nb partial sums by T threads (red: T doubles in shared
+// memory): four chains per thread, then a tree.  All threads call; thread 0 gets it.
+template <int T>
+__device__ __forceinline__ double sum_parts(const double *part, int nb, double *red)
+{
+    const int tid = threadIdx.x;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int k = tid; k < nb; k += 4 * T)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (k + j * T < nb) s[j] = __dadd_rn(s[j], __ldcg(part + k + j * T));
+    red[tid] = __dadd_rn(__dadd_rn(s[0], s[1]), __dadd_rn(s[2], s[3]));
+    __syncthreads();
+    for (int o = T / 2; o > 0; o >>= 1) {
+        if (tid < o) red[tid] = __dadd_rn(red[tid], red[tid + o]);
+        __syncthreads();
+    }
+    return red[0];
+}
+
+// The last of a replica's nb blocks to get here, with all their parts visible,
+// gets true; it leaves the counter at zero.  All threads call; the block's own
+// part was written by thread 0.  The counter is the MD run's own, whose steps
+// follow one another.
+__device__ __forceinline__ bool last_block(unsigned *arrived, int nb)
+{
+    __shared__ int last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(arrived, 1u) == (unsigned)nb - 1u;
+        if (last) {
+            *arrived = 0;
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    return last != 0;
+}
+
 // The end of a step for a block: its sum of v^2 (every thread's share), and by
 // the replica's last block the thermostat; clears the cell counts for the next step.
 template <int T>
@@ -113,7 +152,7 @@ __device__ void md_end_step(const DevState &d, const MdDev &m, int r, int b0, in
         for (int k = 1; k < T / 32; ++k) v2 = __dadd_rn(v2, red[k]);
         m.part[blockIdx.x] = v2;
     }
-    if (!last_block(d.arrived + r, nb)) return;
+    if (!last_block(m.arrived + r, nb)) return;
     v2 = sum_parts<T>(m.part + b0, nb, red);
     if (threadIdx.x == 0) md_thermostat(d, m, r, v2, true);
 }

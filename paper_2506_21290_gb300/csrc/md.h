@@ -22,6 +22,7 @@ struct MdDev {
     const double *Q;   // per replica: thermostat mass g T tau^2, g = 3 N
     Units units;       // blocks of the force kernel: kMdWarps cells (FP64), or 32 records (FP32)
     double *part;      // per block: partial sum of v^2
+    unsigned *arrived; // per replica: blocks that have written theirs (zero between steps)
     int fp32_forces;   // 1: pair forces in FP32 (velocities, positions and thermostat stay FP64)
     double dt;
     double hdt;        // dt / 2

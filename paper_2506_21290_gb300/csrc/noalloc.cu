@@ -49,8 +49,7 @@ constexpr size_t kOffModel = al256(kOffCtr + sizeof(RepCtr));
 constexpr size_t kOffMix = al256(kOffModel + sizeof(ModelDev));
 constexpr size_t kOffActOff = al256(kOffMix + sizeof(MixDev));
 constexpr size_t kOffErr = al256(kOffActOff + 2 * sizeof(int));
-constexpr size_t kOffArrived = al256(kOffErr + sizeof(int));
-constexpr size_t kOffRepOfSite = al256(kOffArrived + sizeof(unsigned));
+constexpr size_t kOffRepOfSite = al256(kOffErr + sizeof(int));
 constexpr size_t kOffRec0 = al256(kOffRepOfSite + sizeof(int) * kMaxSites);
 constexpr size_t kOffRec1 = al256(kOffRec0 + sizeof(int4) * kMaxSites);
 constexpr size_t kOffCount = al256(kOffRec1 + sizeof(int4) * kMaxSites);
@@ -109,7 +108,6 @@ __global__ void noalloc_init_kernel(Header hd, unsigned char *base, int n_sites)
         ((int *)(base + kOffActOff))[0] = hd.act_off[0];
         ((int *)(base + kOffActOff))[1] = hd.act_off[1];
         *(int *)(base + kOffErr) = 0;
-        *(unsigned *)(base + kOffArrived) = 0;
     }
     int *rep_of_site = (int *)(base + kOffRepOfSite);
     for (int i = threadIdx.x; i < n_sites; i += blockDim.x) rep_of_site[i] = 0;
@@ -225,7 +223,6 @@ extern "C" int mc_energy_noalloc(double L, int n_mol, const uint32_t *dev_q, con
     d.cell_start = (int *)(base + kOffStart);
     d.cell_of = (int *)(base + kOffCellOf);
     d.slot_of = (int *)(base + kOffSlotOf);
-    d.arrived = (unsigned *)(base + kOffArrived);
     d.cells.n = n_cells / (kEnergyWarps * walk_cells(n_sites, n_cells));
     double *e_part = (double *)(base + kOffESite);   // per-block partial sums
 

@@ -174,42 +174,4 @@ __host__ __device__ constexpr int walk_cells(int n_sites, int n_cells)
     return n_sites >= 14 * n_cells ? 1 : (n_sites >= 8 * n_cells ? 2 : 4);
 }
 
-// Fixed-order sum over nb partial sums by T threads (red: T doubles in shared
-// memory): four chains per thread, then a tree.  All threads call; thread 0 gets it.
-template <int T>
-__device__ __forceinline__ double sum_parts(const double *part, int nb, double *red)
-{
-    const int tid = threadIdx.x;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k = tid; k < nb; k += 4 * T)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (k + j * T < nb) s[j] = __dadd_rn(s[j], __ldcg(part + k + j * T));
-    red[tid] = __dadd_rn(__dadd_rn(s[0], s[1]), __dadd_rn(s[2], s[3]));
-    __syncthreads();
-    for (int o = T / 2; o > 0; o >>= 1) {
-        if (tid < o) red[tid] = __dadd_rn(red[tid], red[tid + o]);
-        __syncthreads();
-    }
-    return red[0];
-}
-
-// The last of a replica's nb blocks to get here, with all their parts visible,
-// gets true; it leaves the counter at zero.  All threads call; the block's own
-// part was written by thread 0.
-__device__ __forceinline__ bool last_block(unsigned *arrived, int nb)
-{
-    __shared__ int last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(arrived, 1u) == (unsigned)nb - 1u;
-        if (last) {
-            *arrived = 0;
-            __threadfence();
-        }
-    }
-    __syncthreads();
-    return last != 0;
-}
-
 }  // namespace flipmc
