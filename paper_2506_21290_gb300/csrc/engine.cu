@@ -1057,19 +1057,21 @@ int mc_autotune(mc_handle *h, int n_sweeps, const double *T, const mc_move_mix *
     int rc = check_mix(mix);
     if (rc) return rc;
     if ((rc = set_device(h))) return rc;
-    // device snapshot of everything a sweep changes
+    // device snapshot of everything a sweep changes that outlives it (the
+    // cells' extents too: the energy, the virial and MD read the records by them)
     const size_t n = (size_t)h->n_sites, R = (size_t)h->n_rep;
     const size_t b_rec = sizeof(int4) * n, b_img = sizeof(int) * 3 * n, b_e = sizeof(double) * R,
-                 b_st = sizeof(unsigned long long) * STAT_N * R, b_ct = sizeof(RepCtr) * R;
+                 b_st = sizeof(unsigned long long) * STAT_N * R, b_ct = sizeof(RepCtr) * R,
+                 b_cs = sizeof(int) * ((size_t)h->n_cells + 1);
     unsigned char *snap = nullptr;
-    CUDA_TRY(cudaMalloc(&snap, b_rec + b_img + b_e + b_st + b_ct));
+    CUDA_TRY(cudaMalloc(&snap, b_rec + b_img + b_e + b_st + b_ct + b_cs));
     const int cur0 = h->cur, W0 = h->wpb;
     const bool p0 = h->pgrid > 0;
     auto copy_all = [&](bool save) {
-        void *dev[5] = {h->ds.rec[cur0], h->ds.img, h->ds.e_run, h->ds.stats, h->ds.ctr};
-        const size_t sz[5] = {b_rec, b_img, b_e, b_st, b_ct};
+        void *dev[6] = {h->ds.rec[cur0], h->ds.img, h->ds.e_run, h->ds.stats, h->ds.ctr, h->ds.cell_start};
+        const size_t sz[6] = {b_rec, b_img, b_e, b_st, b_ct, b_cs};
         size_t off = 0;
-        for (int k = 0; k < 5; ++k) {
+        for (int k = 0; k < 6; ++k) {
             if (save) cudaMemcpyAsync(snap + off, dev[k], sz[k], cudaMemcpyDeviceToDevice, h->stream);
             else cudaMemcpyAsync(dev[k], snap + off, sz[k], cudaMemcpyDeviceToDevice, h->stream);
             off += sz[k];
