@@ -35,6 +35,8 @@ thread_local std::string g_err;
 int fail(int code, const std::string &msg)
 {
     g_err = msg;
+    // (an error that this call reports is not one of the next call's launches)
+    if (code == MC_ERR_CUDA) cudaGetLastError();
     return code;
 }
 
