@@ -471,10 +471,12 @@ int pack_records(mc_handle *h, const double *xyz, const uint32_t *qfix, const in
 // The results of one call, in page-locked memory: copies enqueued on the
 // stream, then finish(), which also fetches the device's error word and waits, once
 // (a copy to pageable memory and a wait for each result cost 5 to 10 us apiece).
+// When a copy or the wait fails, the memory holds an earlier call's results:
+// arrived() tells whether there is anything to hand over.
 class Results {
 public:
     Results(mc_handle *h, size_t bytes) : h_(h), base_((unsigned char *)h->results.get(bytes + 256)) {}
-    // n values from device memory; valid after finish()
+    // n values from device memory; valid once they have arrived
     template <class T>
     const T *get(const T *dev, size_t n)
     {
@@ -488,8 +490,11 @@ public:
     {
         CUDA_TRY(failed_);
         CUDA_TRY(cudaStreamSynchronize(h_->stream));
+        arrived_ = true;
         return MC_OK;
     }
+    bool arrived() const { return arrived_; }
+    // (an error that the device reports comes with its results)
     int finish()
     {
         const int *err = get(h_->ds.err, 1);
@@ -507,6 +512,7 @@ private:
     unsigned char *base_;
     size_t used_ = 0;
     cudaError_t failed_ = cudaSuccess;
+    bool arrived_ = false;
 };
 
 int check_device_errors(mc_handle *h) { return Results(h, 0).finish(); }
@@ -1160,6 +1166,7 @@ int mc_energy(mc_handle *h, double *E_out)
     Results res(h, sizeof(double) * h->n_rep);
     const double *e = res.get(h->d_e_out, h->n_rep);
     rc = res.finish();
+    if (!res.arrived()) return rc;
     std::memcpy(E_out, e, sizeof(double) * h->n_rep);
     return rc;
 }
@@ -1176,6 +1183,7 @@ int mc_pressure(mc_handle *h, const double *T, double *out)
     Results res(h, sizeof(double) * h->n_rep);
     const double *w = res.get(h->d_e_out, h->n_rep);
     rc = res.finish();
+    if (!res.arrived()) return rc;
     for (int r = 0; r < h->n_rep; ++r) {
         const double V = h->reps[r].L * h->reps[r].L * h->reps[r].L;
         out[2 * r] = w[r];
@@ -1228,6 +1236,7 @@ int mc_structure_factor(mc_handle *h, const double *qvec, int n_q, double *out)
     Results res(h, b_out);
     const double *got = res.get(dout, (size_t)n_q * R);
     rc = res.finish();
+    if (!res.arrived()) return rc;
     std::memcpy(out, got, b_out);
     return rc;
 }
@@ -1253,6 +1262,7 @@ int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, dou
     Results res(h, sizeof(unsigned long long) * n);
     const unsigned long long *got = res.get(dc, n);
     rc = res.finish();
+    if (!res.arrived()) return rc;
     std::memcpy(counts, got, sizeof(unsigned long long) * n);
     if (g) {
         // g(r) at the bin centres: 2 counts / (N rho shell volume), rho = N / V
@@ -1306,7 +1316,8 @@ int mc_state(mc_handle *h, double *xyz_out, int32_t *types_out, mc_stats *stats_
         dr = res.get(h->d_drift, 2 * R);
     }
     if (!rec && !stats_out) return MC_OK;
-    if ((rc = res.finish()) && rec) return rc;
+    rc = res.finish();
+    if (!res.arrived() || (rc && rec)) return rc;
     if (rec) {
         // on host threads, each taking a run of record slots (a replica's
         // records fill the slots of its sites; each record writes its own site)
@@ -1974,6 +1985,7 @@ int mc_md_state(mc_handle *h, double *v_out, double *out)
     const double *v = res.get(h->md.dev.v, nv), *xi = res.get(h->md.dev.xi, R), *eta = res.get(h->md.dev.eta, R),
                  *U = res.get(h->d_e_out, R);
     rc = res.finish();
+    if (!res.arrived()) return rc;
     if (v_out) std::memcpy(v_out, v, sizeof(double) * nv);
     for (int r = 0; r < R; ++r) {
         double K = 0.0;
