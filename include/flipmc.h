@@ -198,8 +198,10 @@ typedef struct {
  * replica, then site, then bond order is reported.  Host work: the packing and
  * validation of more than 8192 molecules runs on up to 16 host threads started
  * and joined inside the call; the handle keeps a page-locked staging buffer
- * (16 to 28 bytes per atom) for the state's copies.  Model: Sec. II.A; schedule as
- * described above.
+ * (16 to 28 bytes per atom) for the state's copies, and for its read-outs
+ * page-locked memory (up to 24 bytes per atom, or 64 MB where the size is the
+ * caller's choice) and at most 64 MB of device workspace.  Model: Sec. II.A;
+ * schedule as described above.
  */
 int mc_create(mc_handle **out, double L, int n_mol, const double *xyz, const int32_t *types,
               const mc_params *params, const mc_options *opts);

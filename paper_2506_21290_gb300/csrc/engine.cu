@@ -50,6 +50,10 @@ int fail(int code, const std::string &msg)
 const double kCbrt2 = 0x1.428a2f98d728bp+0;   // double nearest 2^(1/3)
 const double kTwo32 = 4294967296.0;
 const int kMaxPersistentBlocks = 8192;
+// what a handle keeps of a workspace between calls, and the largest result that
+// goes through page-locked memory when its size is the caller's choice (n_q or
+// n_bins times the replicas); a larger one is copied to the caller's array directly
+const size_t kKeep = (size_t)64 << 20;
 
 // x -> floor(frac(x / L) * 2^32), the library's quantisation of positions
 uint32_t quantize(double x, double L)
@@ -124,6 +128,7 @@ struct mc_handle {
         void *pin = nullptr;
         size_t bytes = 0;
         std::vector<unsigned char> pageable;
+        // null when there is no host memory at all (no exception leaves a C entry)
         void *get(size_t n)
         {
             if (pin && bytes >= n) return pin;
@@ -134,7 +139,11 @@ struct mc_handle {
             }
             pin = nullptr;
             cudaGetLastError();
-            pageable.resize(n);
+            try {
+                pageable.resize(n);
+            } catch (const std::exception &) {
+                return nullptr;
+            }
             return pageable.data();
         }
         void release()
@@ -144,9 +153,13 @@ struct mc_handle {
             bytes = 0;
         }
     } staging, results;
-    void *host_buf(size_t bytes) { return staging.get(bytes); }
+    int host_buf(size_t n, void **out)
+    {
+        *out = staging.get(n);
+        return *out ? MC_OK : fail(MC_ERR_CUDA, "no host memory for the copies");
+    }
     // device workspace of the analysis calls, grown on demand and kept with the
-    // handle; a call lays its arrays out in it anew
+    // handle up to kKeep bytes; a call lays its arrays out in it anew
     void *work = nullptr;
     size_t work_bytes = 0;
     int need_work(size_t bytes)
@@ -165,6 +178,14 @@ struct mc_handle {
         }
         work_bytes = bytes;
         return MC_OK;
+    }
+    // at the end of a call that has waited for the stream
+    void trim_work()
+    {
+        if (work_bytes <= kKeep) return;
+        cudaFree(work);
+        work = nullptr;
+        work_bytes = 0;
     }
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
@@ -480,11 +501,21 @@ public:
     template <class T>
     const T *get(const T *dev, size_t n)
     {
+        if (!base_) {
+            failed_ = cudaErrorMemoryAllocation;
+            return nullptr;
+        }
         T *to = (T *)(base_ + used_);
         used_ += (n * sizeof(T) + 15) & ~(size_t)15;
+        copy(to, dev, n);
+        return to;
+    }
+    // the same into the caller's memory (too large to be kept)
+    template <class T>
+    void copy(T *to, const T *dev, size_t n)
+    {
         const cudaError_t e = cudaMemcpyAsync(to, dev, n * sizeof(T), cudaMemcpyDeviceToHost, h_->stream);
         if (failed_ == cudaSuccess) failed_ = e;
-        return to;
     }
     int wait()
     {
@@ -516,6 +547,24 @@ private:
 };
 
 int check_device_errors(mc_handle *h) { return Results(h, 0).finish(); }
+
+// One result of n values, whose number is the caller's choice, from the
+// workspace into the caller's array: the end of an analysis call.
+template <class T>
+int hand_over(mc_handle *h, T *out, const T *dev, size_t n, bool *arrived = nullptr)
+{
+    const size_t bytes = sizeof(T) * n;
+    const bool direct = bytes > kKeep;
+    Results res(h, direct ? 0 : bytes);
+    const T *got = nullptr;
+    if (direct) res.copy(out, dev, n);
+    else got = res.get(dev, n);
+    const int rc = res.finish();
+    if (res.arrived() && !direct) std::memcpy(out, got, bytes);
+    if (arrived) *arrived = res.arrived();
+    h->trim_work();
+    return rc;
+}
 
 // energy of each replica into h->d_e_out (device)
 int enqueue_energy(mc_handle *h)
@@ -845,10 +894,12 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         mc_destroy(h);
         return fail(MC_ERR_INVALID_ARG, "persistent sweeps need cooperative launch support");
     }
-    int4 *rec = (int4 *)h->host_buf(sizeof(int4) * (size_t)h->n_sites);
+    int4 *rec = nullptr;
+    rc = h->host_buf(sizeof(int4) * (size_t)h->n_sites, (void **)&rec);
     // room for the per-particle results and wavevector tables of the analysis calls
     h->results.get(((size_t)64 << 10) + sizeof(double) * ((size_t)h->n_sites + 2 * (size_t)M_tot + 3 * (size_t)n_rep));
-    rc = h->need_work(std::min<size_t>((size_t)8 << 20, ((size_t)64 << 10) + 512 * sizeof(Turns) * (size_t)n_rep));
+    if (rc == MC_OK)
+        rc = h->need_work(std::min<size_t>((size_t)8 << 20, ((size_t)64 << 10) + 512 * sizeof(Turns) * (size_t)n_rep));
     if (rc == MC_OK) rc = pack_records(h, xyz, nullptr, types, rec);
     if (rc == MC_OK) rc = rebuild_and_reset(h, rec);
     if (rc) {
@@ -1233,12 +1284,7 @@ int mc_structure_factor(mc_handle *h, const double *qvec, int n_q, double *out)
         launch_sq(h->ds, h->cur, turns, n, max_sites, part, dout + k, n_q, h->stream);
     }
     CUDA_TRY(cudaGetLastError());
-    Results res(h, b_out);
-    const double *got = res.get(dout, (size_t)n_q * R);
-    rc = res.finish();
-    if (!res.arrived()) return rc;
-    std::memcpy(out, got, b_out);
-    return rc;
+    return hand_over(h, out, dout, (size_t)n_q * R);
 }
 
 int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, double *g)
@@ -1259,12 +1305,9 @@ int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, dou
     CUDA_TRY(cudaMemsetAsync(dc, 0, sizeof(unsigned long long) * n, h->stream));
     launch_pair_hist(h->ds, h->cur, max_sites, dr, n_bins, dc, h->stream);
     CUDA_TRY(cudaGetLastError());
-    Results res(h, sizeof(unsigned long long) * n);
-    const unsigned long long *got = res.get(dc, n);
-    rc = res.finish();
-    if (!res.arrived()) return rc;
-    std::memcpy(counts, got, sizeof(unsigned long long) * n);
-    if (g) {
+    bool arrived;
+    rc = hand_over(h, (unsigned long long *)counts, dc, n, &arrived);
+    if (g && arrived) {
         // g(r) at the bin centres: 2 counts / (N rho shell volume), rho = N / V
         const double pi = 3.14159265358979323846;
         for (int r = 0; r < h->n_rep; ++r) {
@@ -1284,7 +1327,9 @@ int mc_pair_histogram(mc_handle *h, double dr, int n_bins, uint64_t *counts, dou
 static int fetch_records(mc_handle *h, const int4 **rec, const int **img)
 {
     const size_t n = (size_t)h->n_sites;
-    unsigned char *buf = (unsigned char *)h->host_buf(sizeof(int4) * n + (img ? sizeof(int) * 3 * n : 0));
+    unsigned char *buf = nullptr;
+    const int rc = h->host_buf(sizeof(int4) * n + (img ? sizeof(int) * 3 * n : 0), (void **)&buf);
+    if (rc) return rc;
     CUDA_TRY(cudaMemcpyAsync(buf, h->ds.rec[h->cur], sizeof(int4) * n, cudaMemcpyDeviceToHost, h->stream));
     if (img)
         CUDA_TRY(cudaMemcpyAsync(buf + sizeof(int4) * n, h->ds.img, sizeof(int) * 3 * n, cudaMemcpyDeviceToHost,
@@ -1391,7 +1436,8 @@ int mc_set_state(mc_handle *h, const double *xyz, const int32_t *types)
     if (!h || !xyz || !types) return fail(MC_ERR_INVALID_ARG, "NULL argument");
     int rc = set_device(h);
     if (rc) return rc;
-    int4 *rec = (int4 *)h->host_buf(sizeof(int4) * (size_t)h->n_sites);
+    int4 *rec = nullptr;
+    if ((rc = h->host_buf(sizeof(int4) * (size_t)h->n_sites, (void **)&rec))) return rc;
     if ((rc = pack_records(h, xyz, nullptr, types, rec))) return rc;
     return rebuild_and_reset(h, rec);
 }
@@ -1401,7 +1447,8 @@ int mc_set_state_fixed(mc_handle *h, const uint32_t *q, const int64_t *X, const 
     if (!h || !q || !types) return fail(MC_ERR_INVALID_ARG, "NULL argument");
     int rc = set_device(h);
     if (rc) return rc;
-    int4 *rec = (int4 *)h->host_buf(sizeof(int4) * (size_t)h->n_sites);
+    int4 *rec = nullptr;
+    if ((rc = h->host_buf(sizeof(int4) * (size_t)h->n_sites, (void **)&rec))) return rc;
     if ((rc = pack_records(h, nullptr, q, types, rec))) return rc;
     if (!X) return rebuild_and_reset(h, rec);
     std::vector<int> img(3 * (size_t)h->n_sites);
@@ -1465,7 +1512,8 @@ int mc_observables(mc_handle *h, const double *qvec_atom, int n_qa, const double
     Turns *ta = (Turns *)h->work, *tc = ta + R * n_qa;
     double *dqa = (double *)(tc + R * n_qc), *dqc = dqa + 3 * n_qa;
     const size_t b_qa = sizeof(double) * 3 * n_qa, b_qc = sizeof(double) * 3 * n_qc;
-    unsigned char *hq = (unsigned char *)h->host_buf(b_qa + b_qc);
+    unsigned char *hq = nullptr;
+    if ((rc = h->host_buf(b_qa + b_qc, (void **)&hq))) return rc;
     std::memcpy(hq, qvec_atom, b_qa);
     std::memcpy(hq + b_qa, qvec_cm, b_qc);
     CUDA_TRY(cudaMemcpyAsync(dqa, hq, b_qa + b_qc, cudaMemcpyHostToDevice, h->stream));
