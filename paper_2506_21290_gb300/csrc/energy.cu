@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(32 * kEnergyWarps) pair_energy_kernel(DevState
     EnergyWalk<VIRIAL> p{md, quantum2(ri.h), 6.0 * md.e4, walk[w].ring, bond_r2[w], bond_ab[w], lane};
     int head = 0, tail = 0;
     for (int k = 0; k < per; ++k)
-        walk_cell<true>(d, ri, md, d.rec[buf], c0 + w * per + k, lane, walk[w], head, tail, p);
+        walk_cell<true, false>(d, ri, md, d.rec[buf], c0 + w * per + k, lane, walk[w], head, tail, p);
     if (tail > head) p.eval(head, tail - head);
     if (p.bond_tail > p.bond_head) p.bonds(p.bond_tail - p.bond_head);
     double v = p.acc;

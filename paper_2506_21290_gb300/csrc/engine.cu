@@ -1945,7 +1945,7 @@ int mc_md_setup(mc_handle *h, double dt, double tau_T, const double *T, const do
     const bool fp32 = force_precision == MC_PREC_FP32;
     const HostUnits units = make_units(h->reps, [&](const RepInfo &ri) {
         return fp32 ? std::make_pair(std::make_pair(ri.site_off, ri.n_sites), 32)
-                    : std::make_pair(std::make_pair(ri.cell_off, ri.nc * ri.nc * ri.nc), kMdWarps);
+                    : std::make_pair(std::make_pair(0, md_warps(ri.n_sites, ri.nc * ri.nc * ri.nc).n), kMdWarps);
     });
     const size_t nu = units.unit.size();
     double *bufs[10] = {};

@@ -264,7 +264,19 @@ __global__ void __launch_bounds__(32 * kMdWarps, 4) md_force64_kernel(DevState d
     const RepInfo ri = d.rep[u.x];
     ForceWalk p{ri, *d.model, m, walk[w].ring, list[w], first[w], lane, quantum2(ri.h), m.scale[u.x], end_step != 0};
     int head = 0, tail = 0;
-    walk_cell<false>(d, ri, *d.model, d.rec[buf], u.y + w, lane, walk[w], head, tail, p);
+    const int n_cells = ri.nc * ri.nc * ri.nc;
+    const MdWarps mw = md_warps(ri.n_sites, n_cells);
+    const int id = u.y + w;        // warp of the replica
+    const int cell = id / mw.slices, c0 = ri.cell_off + cell * mw.cells;
+    unsigned todo = cell < n_cells ? 1u : 0u;   // cells c0 + bit
+    if (mw.cells > 1) {
+        const int c = c0 + lane;
+        const bool full = lane < mw.cells && c < ri.cell_off + n_cells && d.cell_start[c + 1] > d.cell_start[c];
+        todo = __ballot_sync(0xffffffffu, full);
+    }
+    for (; todo != 0; todo &= todo - 1)
+        walk_cell<false, true>(d, ri, *d.model, d.rec[buf], c0 + __ffs(todo) - 1, lane, walk[w], head, tail, p,
+                               id - cell * mw.slices, mw.slices);
     const int b0 = m.units.rep0[u.x];
     if (end_step) md_end_step<32 * kMdWarps>(d, m, u.x, b0, m.units.rep0[u.x + 1] - b0, p.v2, red);
 }

@@ -64,20 +64,22 @@ __device__ __forceinline__ double walk_rcp(double x)
 }
 
 // Pairs of cell c's atoms with the atoms of its neighbourhood (HALF: those of a
-// larger site index, so that a walk over all cells meets each pair once).  The
+// larger site index, so that a walk over all cells meets each pair once).  SLICED:
+// of the cell's atoms in groups of 32, number `slice` and every n_slices-th after it.
+// The
 // ring holds positions head .. tail - 1, fewer than 32 between calls of P:
 // P: own(i0, ni, rec)   the next (at most 32) own atoms; lane i holds atom i's record
 //    atom(i, tail)      own atom i's pairs begin at this position
 //    eval(at, 32)       evaluate the pairs at positions at, at + 1, ... (whole warp)
 //    part(head, tail)   no more pairs of these atoms with this part of the candidates
 //    done()             these own atoms are finished
-template <bool HALF, class P>
+template <bool HALF, bool SLICED, class P>
 __device__ __forceinline__ void walk_cell(const DevState &d, const RepInfo &ri, const ModelDev &md, const int4 *rec, int c,
-                                          int lane, WalkSmem &sm, int &head, int &tail, P &p)
+                                          int lane, WalkSmem &sm, int &head, int &tail, P &p, int slice = 0, int n_slices = 1)
 {
     constexpr unsigned FULL_WARP = 0xffffffffu;
     const int s0 = d.cell_start[c], n = d.cell_start[c + 1] - s0;
-    if (n == 0) return;
+    if (n <= (SLICED ? 32 * slice : 0)) return;
     const int nc = ri.nc, cl = c - ri.cell_off;
     const int cx = cl % nc, cy = (cl / nc) % nc, cz = cl / (nc * nc);
     const bool small = nc == 2;
@@ -110,7 +112,7 @@ __device__ __forceinline__ void walk_cell(const DevState &d, const RepInfo &ri, 
     // cutoffs of the nine type pairs in fixed-point units squared, one per lane
     const float cut = lane < 9 ? md.rc2f[lane] * 1.00002f / ri.hf / ri.hf : 0.f;
     const unsigned lt = (1u << lane) - 1u;
-    for (int i0 = 0; i0 < n; i0 += 32) {
+    for (int i0 = SLICED ? 32 * slice : 0; i0 < n; i0 += SLICED ? 32 * n_slices : 32) {
         const int ni = min(32, n - i0);
         const int4 own = rec[s0 + i0 + min(lane, ni - 1)];
         p.own(i0, ni, own);
