@@ -1182,10 +1182,8 @@ __device__ Res evaluate(const CellCtx &cx, const Group &G, const WarpScr &S, Nea
     }
     if (W > 1 && lane == 0) {
         // positions the move reads or writes, for the conflict test of the commit
-        // (a move that breaks a bond too: an earlier attempt does not change its
-        // refusal, but may change its count of pairs in range)
         int na = 0;
-        if (status == MC_ST_EVALUATED || status == MC_ST_BOND_BREAK) {
+        if (status == MC_ST_EVALUATED) {
 #pragma unroll
             for (int s = 0; s < 3; ++s) {
                 if (s < nmv) {
