@@ -47,9 +47,11 @@ __device__ __forceinline__ double walk_ln(double y)
 // (No counter tells a last block to add the blocks' sums: mc_energy_device is
 // asynchronous, so two of these may overlap on two streams, or in two replayed
 // graphs, with one handle's workspace.  Both write the same numbers to it.)
-// Energy of 24000 atoms 41 us (62 with the sum over cells, when every lane of a
-// warp walked a neighbour cell and bonds shared the batches), of 192000 atoms
-// 133 (290), of 256 replicas with 823000 atoms 505 (1161).
+// Energy of 24000 atoms 42 us (62 when every lane of a warp walked a neighbour
+// cell and bonds shared the batches), of 192000 atoms 124 (290), of 256 replicas
+// with 823000 atoms 494 (1161), both kernels.  96 registers with 52 bytes of
+// spills: without them at 116 registers the last two take 133 and 559, and at 92
+// registers 122 and 496.
 template <bool VIRIAL>
 struct EnergyWalk {
     const ModelDev &md;

@@ -222,7 +222,7 @@ struct mc_handle {
     int *d_rep_of_site = nullptr;
     int *d_act_off = nullptr;
     int2 *d_act_slot = nullptr;
-    double *d_e_site = nullptr;          // per-cell (or per-site) FP64 partial sums
+    double *d_parts = nullptr;           // FP64 partial sums of an energy walk, one per block
     double *d_e_out = nullptr;
     long long *d_X = nullptr;
     int *d_types = nullptr;
@@ -569,7 +569,7 @@ int hand_over(mc_handle *h, T *out, const T *dev, size_t n, bool *arrived = null
 // energy of each replica into h->d_e_out (device)
 int enqueue_energy(mc_handle *h)
 {
-    launch_energy(h->ds, h->cur, h->d_e_site, h->d_e_out, h->stream);
+    launch_energy(h->ds, h->cur, h->d_parts, h->d_e_out, h->stream);
     CUDA_TRY(cudaGetLastError());
     return MC_OK;
 }
@@ -726,8 +726,7 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         // kernels use them (one rounding per operation)
         float rc2max = 0.f;
         for (int k = 0; k < 9; ++k) rc2max = std::fmax(rc2max, h->model_host.rc2f[k]);
-        ri.pre_r2 = rc2max * 1.01f;
-        ri.r2q = ri.pre_r2 / ri.h2f;
+        ri.r2q = rc2max * 1.01f / ri.h2f;
         ri.rconf = rc2max * 1.0201f / ri.h2f;
         h->reps.push_back(ri);
         for (int i = 0; i < ri.n_sites; ++i) rep_of_site.push_back(r);
@@ -827,7 +826,7 @@ int create_impl(mc_handle **out, int n_rep, const double *L, const int32_t *n_mo
         (rc = h->alloc(&cs, h->n_cells + 1)) || (rc = h->alloc(&co, h->n_sites)) || (rc = h->alloc(&so, h->n_sites)) ||
         (rc = h->alloc(&img, 3 * (size_t)h->n_sites)) || (rc = h->alloc(&cde, h->n_cells)) ||
         (rc = h->alloc(&stats, (size_t)STAT_N * n_rep)) || (rc = h->alloc(&erun, n_rep)) ||
-        (rc = h->alloc(&err, 1)) || (rc = h->alloc(&h->d_e_site, std::max(h->n_sites, h->n_cells))) ||
+        (rc = h->alloc(&err, 1)) || (rc = h->alloc(&h->d_parts, cell_units.unit.size())) ||
         (rc = h->alloc(&h->d_e_out, n_rep)) || (rc = h->alloc(&h->d_X, 3 * (size_t)h->n_sites)) ||
         (rc = h->alloc(&h->d_types, h->n_sites)) || (rc = h->alloc(&h->obs.X0, 3 * (size_t)h->n_sites)) ||
         (rc = h->alloc(&h->obs.kref, M_tot)) || (rc = h->alloc(&h->obs.u0, 3 * (size_t)M_tot)) ||
@@ -1229,7 +1228,7 @@ int mc_pressure(mc_handle *h, const double *T, double *out)
         if (!(T[r] > 0.0) || !std::isfinite(T[r])) return fail(MC_ERR_INVALID_ARG, "temperature must be positive");
     int rc = set_device(h);
     if (rc) return rc;
-    launch_virial(h->ds, h->cur, h->d_e_site, h->d_e_out, h->stream);
+    launch_virial(h->ds, h->cur, h->d_parts, h->d_e_out, h->stream);
     CUDA_TRY(cudaGetLastError());
     Results res(h, sizeof(double) * h->n_rep);
     const double *w = res.get(h->d_e_out, h->n_rep);

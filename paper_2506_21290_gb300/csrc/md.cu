@@ -10,13 +10,13 @@
 // K is the kinetic energy sum v^2 / 2 over the replica, in a fixed order.  The
 // conserved quantity is K + U + Q xi^2 / 2 + g T eta.
 //
-// A step is five kernels: the move (kick, drift and the count of the cell list),
-// its scan, scatter and order, and the forces, whose blocks end the step for
-// their atoms.  The kinetic energy at the start of a step is the one at the
-// end of the step before, so the block that is the last of its replica to
-// finish takes both thermostat half steps.  (As thirteen kernels, with K
-// summed twice, the parts beside the forces took 45 us a step at 1000
-// molecules and 70 at 64000.)
+// A step is five kernels, seven above 8192 cells: the move (kick, drift and the
+// count of the cell list), its scan (one kernel or three), scatter and order, and
+// the forces, whose blocks end the step for their atoms.  The kinetic energy at
+// the start of a step is the one at the end of the step before, so the block that
+// is the last of its replica to finish takes both thermostat half steps.  (As
+// thirteen kernels, with K summed twice, the parts beside the forces took 45 us a
+// step at 1000 molecules and 70 at 64000.)
 #include "cell_list.h"
 #include "cell_list_dev.cuh"
 #include "flipmc_device.cuh"

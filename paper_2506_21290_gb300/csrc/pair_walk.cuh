@@ -52,8 +52,9 @@ __device__ __forceinline__ double walk_r2(const int4 &e, const Quantum2 &q)
 }
 
 // 1 / x to about one unit: an FP32 reciprocal (2^-21) and one third-order
-// Newton step (the error's cube is 2^-63), four FP64 operations in a chain
-// where a division takes eleven.  Outside FP32's range, the division.
+// Newton step (the error's cube is 2^-63): three FP64 operations one after the
+// other, 64 cycles each here, where a division takes 564.  Outside FP32's range,
+// the division.
 __device__ __forceinline__ double walk_rcp(double x)
 {
     const float f = (float)x;
@@ -66,8 +67,7 @@ __device__ __forceinline__ double walk_rcp(double x)
 // Pairs of cell c's atoms with the atoms of its neighbourhood (HALF: those of a
 // larger site index, so that a walk over all cells meets each pair once).  SLICED:
 // of the cell's atoms in groups of 32, number `slice` and every n_slices-th after it.
-// The
-// ring holds positions head .. tail - 1, fewer than 32 between calls of P:
+// The ring holds positions head .. tail - 1, fewer than 32 between calls of P:
 // P: own(i0, ni, rec)   the next (at most 32) own atoms; lane i holds atom i's record
 //    atom(i, tail)      own atom i's pairs begin at this position
 //    eval(at, 32)       evaluate the pairs at positions at, at + 1, ... (whole warp)
