@@ -582,6 +582,7 @@ def run_native(args):
                "h2d_bytes_per_step": int(16 * N), "d2h_bytes_per_step": int(28 * N + 8 * h.n_rep + 144 * h.n_rep),
                "steps": args.e2e_steps,
                "path": "mc_set_state (host positions) + mc_sweep + mc_energy + mc_state (host positions)"}
+        h.set_stream(stream.cuda_stream)      # the events of --corr and --md are recorded there
 
     if rank != 0:
         if dist is not None:
