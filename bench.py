@@ -44,7 +44,7 @@ L2_FLUSH_BYTES = 256 << 20
 # DRAM bytes (read + write) per launch of the dominant kernel, from one ncu
 # capture of that kernel on that workload; keyed by (workload, kernel, sweeps
 # per launch), so a timed launch that differs from the captured one reports null
-NCU_TRAFFIC = {}
+NCU_TRAFFIC = {("single-8000", "sweep_persistent<FP32,W=2>", 20): 656128 + 257792}
 
 
 def parse():
@@ -344,9 +344,9 @@ def run_corr(h, wl, mix, P, stream, n_events=10):
     cos_per_pair = 3 * len(qa) + len(qc)
     return {"pairs_per_event": P, "event_ms": ev_ms, "sweep_plus_event_ms": with_ev, "sweep_ms": plain,
             "molecule_samples_per_s": P * M / (ev_ms * 1e-3),
-            "fp64_cos_per_s": P * M * cos_per_pair / (ev_ms * 1e-3),
+            "cos_per_s": P * M * cos_per_pair / (ev_ms * 1e-3),
             "what": "per event: gather of the unwrapped positions, F_s (12 q), F_s^cm (8 q), C_2 per molecule "
-                    "for each pair in FP64, fixed-order per-replica sums, one new origin"}
+                    "for each pair (integer cosines, exact sums), fixed-order per-replica sums, one new origin"}
 
 
 def run_md(h, wl, n_steps, stream):
@@ -356,8 +356,8 @@ def run_md(h, wl, n_steps, stream):
     import torch
     T = np.broadcast_to(np.asarray(wl["T"], dtype=np.float64), (h.n_rep,))
     out = {"steps": n_steps,
-           "what": "one step: thermostat half + kick, drift, cell-list rebuild (4 kernels), forces, kick + "
-                   "thermostat half, as five kernels; eight steps per CUDA graph"}
+           "what": "one step: thermostat half + kick, drift, cell-list rebuild, forces, kick + thermostat half, as "
+                   "five kernels (seven above 8192 cells); eight steps per CUDA graph"}
     for prec in ("fp64", "fp32"):
         h.md_setup(0.001, 1.0, T, W.maxwell_velocities(h.N, float(np.mean(T)), 11), force_precision=prec)
         h.md_run(20)                      # warm-up, graphs instantiated
@@ -424,7 +424,8 @@ def kernel_label(precision, info):
 
 def run_fp64_leg(F, wl, mix, sps, steps, warmup, autotune, stream, flush, sms):
     """The same workload from the same start in FP64 oracle-match mode (every
-    Delta E the FP64 ordered sum, decisions bit-exact to the oracle's chain)."""
+    accepted or doubtful attempt decided by the FP64 ordered sum, the others
+    refused by a rigorous FP32 bound; the chain bit-exact to the oracle's)."""
     import torch
     h = F.Handle(wl["L"], wl["xyz"], wl["types"], W.PAPER_POT, precision="fp64", n_mol=wl["n_mol"])
     if autotune > 0:
@@ -450,8 +451,9 @@ def run_fp64_leg(F, wl, mix, sps, steps, warmup, autotune, stream, flush, sms):
            "kernel": kernel_label("fp64", info), "sweep_launch_ms": sweep_ms / steps,
            "schedule": {"warps_per_cell": info["warps_per_cell"],
                         "launch": "persistent" if info.get("launch_mode", 0) != 1 else "graph per sweep"},
-           "what": "FP64 oracle-match mode: every Delta E the FP64 ordered sum (unfused, fixed order), FP64 "
-                   "thresholds; same workload, start and timing as the FP32 line",
+           "what": "FP64 oracle-match mode: attempts that a rigorous FP32 bound does not refuse are decided by the "
+                   "FP64 ordered sum (unfused, fixed order) and FP64 thresholds, the chain of the sum for every "
+                   "attempt; same workload, start and timing as the FP32 line",
            "clocks": clk}
     h.close()
     return out, (ms, att)
@@ -593,9 +595,9 @@ def run_native(args):
     if not args.no_cpu_baseline and world == 1:
         cpu = cpu_baseline(wl, args.workload, args.cpu_seconds, wl["T"] if wl["replicas"] == 1 else None, mix)
     # our kernels per timed step: the sweeps (one persistent launch, or per
-    # sweep 4 cell-list + 8 colour + 1 finalisation kernels in a graph) and the
-    # energy recompute (1 kernel)
-    launches_per_step = (1 if persistent else 13 * sps) + 1
+    # sweep 4 cell-list (6 above 8192 cells) + 8 colour + 1 finalisation kernels
+    # in a graph) and the energy recompute (2 kernels)
+    launches_per_step = (1 if persistent else (13 if info["total_cells"] <= 8192 else 15) * sps) + 2
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_max / args.steps, "higher_is_better": True,
