@@ -21,13 +21,16 @@
  * n atoms running n attempts; a move that would take an atom out of its cell,
  * or that writes an atom outside the active cell, is rejected.  Random numbers
  * are Philox4x32-10 keyed on (seed) and counted on (attempt, cell, sweep), so a
- * run is reproducible bit for bit and independent of the launch layout.
+ * run is reproducible bit for bit, and its states and decisions are independent
+ * of the launch layout (two statistics are not to the last digit: e_run, whose
+ * terms are added in another order, and pair_interactions, see mc_stats).
  *
  * Precision.  MC_PREC_FP64 decides every attempt as Delta E in FP64 with one
  * rounding per operation, summed in a fixed order (moved atom ascending, then
  * partner index ascending), does; it reproduces the library's FP64 reference
- * trajectory, running energy and counters exactly.  An attempt that a rigorous
- * FP32 bound refuses is refused without the sum (a logged sweep sums them all).
+ * trajectory exactly.  An attempt that a rigorous FP32 bound refuses is refused
+ * without the sum, with the state, running energy and counters of the sum for
+ * every attempt (a logged sweep sums them all).
  * MC_PREC_FP32 evaluates pair terms in FP32 and decides in FP32 when
  * |dE32 - threshold| exceeds recheck_gap times the sum of term magnitudes plus
  * the threshold's own error bound (the FP32 decision then equals the FP64 one);
@@ -150,7 +153,11 @@ typedef struct {
     uint64_t pair_interactions; /* pair-potential evaluations inside their range, old
                                    and new configuration counted apart: WCA terms with
                                    r < 2^(1/6) sigma_ab and FENE terms (FP32 mode: the
-                                   FP32 pass; FP64 mode: the FP64 sum)              */
+                                   FP32 pass; FP64 mode: as the FP64 sum counts).  With
+                                   several warps per cell an attempt that breaks a bond
+                                   is counted in the state at the start of its round, so
+                                   the total may be off by a pair in some 10^8 from that
+                                   of one warp per cell                             */
     uint64_t sweeps;
     double e_run;               /* running FP64 energy: initial + sum of accepted dE */
     uint64_t recomputes;        /* FP64 recomputes made by recompute_every           */
@@ -480,7 +487,7 @@ int mc_relaxation_time(int n_lags, const int64_t *lags, const double *values, co
  * forces in FP64, the oracle-parity path) or MC_PREC_FP32 (pair terms and
  * their per-atom sums in FP32, from the exact int32 differences; velocities,
  * positions, the thermostat and energies stay FP64).
- * mc_md_run: n_steps steps, each one CUDA graph.  Asynchronous.
+ * mc_md_run: n_steps steps, in CUDA graphs of eight steps and of one.  Asynchronous.
  * mc_md_state: v_out[3 N] (nullable) and per replica out[5 r + {0..4}] =
  * K, U, xi, eta, and the conserved K + U + Q xi^2/2 + g T eta (K + U without
  * a thermostat).  Synchronous.

@@ -1802,7 +1802,8 @@ template <int W>
 __host__ __device__ constexpr int phase_threads() { return W == 1 ? 32 : block_threads<W>(); }
 
 // One colour phase, one launch: group g of the grid owns active cell g.
-// W = 1 serves large grids (many cells per SM): registers for fifteen resident blocks (128 per thread)
+// W = 1 serves large grids (many cells per SM): registers for fifteen resident blocks (128 per thread; the FP32 kernel
+// spills 16 bytes there)
 template <int PREC, int W>
 __global__ void __launch_bounds__(phase_threads<W>(), W == 1 ? 15 : 1) phase_kernel(DevState d, int buf, int colour,
                                                                                  LogArgs lg)
