@@ -207,6 +207,7 @@ struct mc_handle {
     // molecular dynamics (mc_md_*)
     struct Md {
         bool on = false;
+        bool stale = false;                 // the state has changed since the forces were taken
         MdDev dev{};
         std::vector<double> T, Q;
         std::vector<void *> bufs;
@@ -578,6 +579,7 @@ int rebuild_and_reset(mc_handle *h, const int4 *rec, const std::vector<int> *img
 {
     // upload in site order into the spare buffer, sort into the other
     const int spare = h->cur;
+    h->md.stale = true;
     CUDA_TRY(cudaMemcpyAsync(h->ds.rec[spare], rec, sizeof(int4) * (size_t)h->n_sites, cudaMemcpyHostToDevice,
                              h->stream));
     launch_cell_list(h->ds, spare, spare ^ 1, h->stream);
@@ -980,6 +982,7 @@ static int sweep_impl(mc_handle *h, int n_sweeps, const double *T, const mc_move
     if (rc) return rc;
     if ((rc = set_device(h))) return rc;
     if ((rc = upload_params(h, T, mix, seeds, same))) return rc;
+    if (n_sweeps > 0) h->md.stale = true;
     while (n_sweeps > 0) {
         // the sweeps up to the next periodic FP64 recompute (all of them when off)
         const int chunk =
@@ -1033,6 +1036,7 @@ int mc_sweep_logged(mc_handle *h, int n_sweeps, const double *T, const mc_move_m
     if ((rc = set_device(h))) return rc;
     if ((rc = upload_params(h, T, mix, seeds, false))) return rc;
     if (n_sweeps == 0) return MC_OK;
+    h->md.stale = true;
     uint64_t sweep0 = 0;
     CUDA_TRY(cudaMemcpy(&sweep0, &h->d_ctr[0].sweep, sizeof(uint64_t), cudaMemcpyDeviceToHost));
     const size_t n = (size_t)n_sweeps * (size_t)h->n_sites;
@@ -1064,6 +1068,7 @@ int mc_sweep_timed(mc_handle *h, int n_sweeps, const double *T, const mc_move_mi
     cudaEvent_t ev[4];
     for (auto &e : ev) CUDA_TRY(cudaEventCreate(&e));
     double tot[3] = {0.0, 0.0, 0.0};
+    if (n_sweeps > 0) h->md.stale = true;
     LogArgs none{nullptr, 0, 0};
     for (int s = 0; s < n_sweeps; ++s) {
         cudaEventRecord(ev[0], h->stream);
@@ -1140,6 +1145,7 @@ int mc_autotune(mc_handle *h, int n_sweeps, const double *T, const mc_move_mix *
     // the trial sweeps make no periodic recompute (the drift figures and the
     // recompute count stay as they are)
     const int every0 = h->recompute_every, since0 = h->since_recompute;
+    const bool stale0 = h->md.stale;
     h->recompute_every = 0;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
@@ -1177,6 +1183,7 @@ int mc_autotune(mc_handle *h, int n_sweeps, const double *T, const mc_move_mix *
     copy_all(false);
     h->recompute_every = every0;
     h->since_recompute = since0;
+    h->md.stale = stale0;
     rc = set_schedule(h, bestW, bestP);
     cudaStreamSynchronize(h->stream);
     cudaEventDestroy(e0);
@@ -2000,6 +2007,12 @@ int mc_md_run(mc_handle *h, int n_steps)
     if (n_steps < 0) return fail(MC_ERR_INVALID_ARG, "n_steps < 0");
     int rc = set_device(h);
     if (rc) return rc;
+    // a step begins with the forces of its configuration: the last step's, unless
+    // sweeps or a new state came between
+    if (n_steps > 0 && h->md.stale) {
+        launch_md_forces(md_state(h), h->cur, h->md.dev, h->stream);
+        h->md.stale = false;
+    }
     // each step counts into cell_count and leaves it zero for the next
     if (n_steps > 0) CUDA_TRY(cudaMemsetAsync(h->ds.cell_count, 0, sizeof(int) * h->n_cells, h->stream));
     for (int s = 0; s < n_steps;) {

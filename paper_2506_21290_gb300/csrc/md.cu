@@ -445,6 +445,11 @@ static void launch_forces(const DevState &d, int buf, const MdDev &m, int end_st
 void launch_md_setup(const DevState &d, int buf, const MdDev &m, cudaStream_t st)
 {
     md_start_kernel<<<d.n_rep, 512, 0, st>>>(d, m);
+    launch_md_forces(d, buf, m, st);
+}
+
+void launch_md_forces(const DevState &d, int buf, const MdDev &m, cudaStream_t st)
+{
     launch_forces(d, buf, m, 0, st);
 }
 

@@ -54,6 +54,8 @@ __host__ __device__ inline MdWarps md_warps(int n_sites, int n_cells)
 
 // The forces of the current state and the first thermostat half step of the first step.
 void launch_md_setup(const DevState &d, int buf, const MdDev &m, cudaStream_t st);
+// The forces alone (the velocities and the thermostat go on as they are).
+void launch_md_forces(const DevState &d, int buf, const MdDev &m, cudaStream_t st);
 // One step from the cell-sorted records of buf into buf ^ 1.  cell_count must be zero, and is again afterwards.
 void launch_md_step(const DevState &d, int buf, const MdDev &m, cudaStream_t st);
 
